@@ -78,7 +78,9 @@ typedef struct {
     int spmv_lanes;       /* lanes per row of the light-row SpMV (1,2,4,8,16,32); <= 0: autotune */
     int inner_chunk;      /* chunked mode: inner iterations launched between convergence checks; <= 0: 16 */
     int inner_graph;      /* 1: each inner solve is one CUDA-graph launch whose WHILE node repeats the
-                             iteration until the device-side stopping test fires (no host round trip);
+                             iteration until the device-side stopping test fires (no host round trip),
+                             or, on small graphs without rows above 64 neighbours and with the diagonal
+                             preconditioner, one kernel launch that holds the whole solve;
                              0: chunked launches with a host check after each chunk */
     int reorder;          /* 1: relabel the vertices internally by descending degree (stable), which
                              packs the vectors' entries of high-degree vertices together for cache
@@ -139,7 +141,8 @@ typedef struct {
     long long inner_solves;
     long long spmv_launches;  /* launches of the inner operator's gather kernel (phase 1) */
     double solve_ms;          /* host wall time of the last isira_solve */
-    double inner_phase1_ms;   /* summed device time of the phase-1 gather launches (profiling on only) */
+    double inner_phase1_ms;   /* summed device time of the phase-1 gather launches (profiling on only); in the
+                                 one-launch solve of a small graph, of its gather and row arithmetic */
     long long inner_phase1_timed; /* number of phase-1 gather launches timed */
     long long inner_phase1_csum;  /* sum of the deflation rank c over the timed phase-1 launches */
     long long kernel_launches;    /* kernels launched by the last isira_solve */
@@ -147,7 +150,8 @@ typedef struct {
     int hub_bytes;                /* shared memory of a gather CTA holding hub vector entries */
     long long hub_timeouts;       /* gather CTAs whose staging copy missed its wait limit (the call
                                      that saw one returned ISIRA_ERR_DEVICE_TIMEOUT) */
-    double inner_rows_ms;         /* summed device time of the phase-1 row kernels (profiling on only) */
+    double inner_rows_ms;         /* summed device time of the phase-1 row kernels (profiling on only); in the
+                                     one-launch solve, of its phase-1 sums */
     double inner_phase2_ms;       /* summed device time of the phase-2 kernels (profiling on only) */
     long long w_columns;          /* sum over outer steps of the search-space size k: the columns of
                                      W_k = (L + delta V V^T) U_k that Algorithm 2 as printed recomputes */
@@ -212,8 +216,8 @@ ISIRA_API isira_status isira_eigpairs(isira_handle h, double* h_eigvals, double*
 /* Counters of the handle (see isira_stats). */
 ISIRA_API isira_status isira_get_stats(isira_handle h, isira_stats* out);
 
-/* 1 = time every phase-1 launch with CUDA events during later solves (adds events
- * between launches; results unchanged), 0 = off. */
+/* 1 = time every phase-1 launch with CUDA events during later solves (adds events between launches; the
+ * one-launch solve of a small graph reads the GPU's timer instead; results unchanged), 0 = off. */
 ISIRA_API isira_status isira_set_profiling(isira_handle h, int on);
 
 /* Releases the handle and all its device memory.  NULL is ignored. */

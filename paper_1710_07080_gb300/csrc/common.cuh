@@ -38,6 +38,8 @@ struct HostStatus {
     int eig_path;          // Rayleigh-Ritz: 0 Jacobi, 1 arrowhead, -1 arrowhead refused (run Jacobi)
     int dev_error;         // bit 0: a gather CTA's staging copy missed its wait limit (set by the
                            // device, cleared by the host at the start of each entry point)
+    unsigned long long prof_ns[3];   // profiled one-launch inner solve: nanoseconds in the gather with its
+                           // row arithmetic, the phase-1 sums, phase 2
 };
 
 // ------------------------------------------------------------------ reductions

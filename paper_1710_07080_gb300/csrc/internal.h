@@ -146,6 +146,22 @@ template <typename T> void ml_phase2b(const InnerArgs<T>& a, int init, cudaGraph
                                       cudaStream_t s);
 template <typename T> void ml_phase2c(const InnerArgs<T>& a, int init, cudaStream_t s);
 
+// one-launch inner solve of a small graph (inner_cluster.cu): one thread-block cluster of `ctas` CTAs
+struct ClusterPlan {
+    int ctas = 0;               // 0: the graph does not take this path
+    int threads = 0, cap = 0;   // threads and row slots per CTA
+    int staged = 0;             // every CTA copies z_k whole into its shared memory and gathers from there
+    int smem = 0;               // dynamic shared memory per CTA
+};
+constexpr int64_t kClusterRows32 = 80000, kClusterRows64 = 30720, kClusterLines = 28000;
+constexpr int kClusterRowsPerCta32 = 256, kClusterRowsPerCta64 = 64;
+// scratch: 8 device bytes; synchronises s
+template <typename T>
+void cluster_plan(const RowSched& rs, int64_t sell_total, unsigned long long* scratch, cudaStream_t s, ClusterPlan* out);
+// prep, init, all iterations and the FP64 result (before the back-map) of one diagonally preconditioned solve
+template <typename T>
+cudaError_t cluster_minres(const InnerArgs<T>& a, const ClusterPlan& p, const double* R, const double* rnorm_dev,
+                           double* Z, bool prof, cudaStream_t s);
 
 // ------------------------------------------------------------------ outer loop (FP64)
 struct OuterArgs {

@@ -139,7 +139,9 @@ struct isira_handle_s {
     cudaGraphExec_t ml_graph[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     double* ml_dv = nullptr;          // kCMax: 1 / (lambda_t - sigma + delta) of the deflated directions
     bool use_ml = false;              // inner solves with the multilevel preconditioner
-    int pending_inner_stats = 0;
+    ClusterPlan cl_f, cl_d;           // one-launch inner solve (small graphs), FP32 and FP64
+    int pending_inner_stats = 0;      // launches per iteration of the solve in flight (-1: the one-launch solve)
+    int pending_c = 0;                // its deflation rank
 };
 
 namespace {
@@ -273,8 +275,31 @@ cudaGraphExec_t build_inner_graph(isira_handle h, const InnerArgs<T>& a) {
     return ex;
 }
 
+template <typename T> const ClusterPlan& cluster_of(isira_handle h);
+template <> const ClusterPlan& cluster_of<float>(isira_handle h) { return h->cl_f; }
+template <> const ClusterPlan& cluster_of<double>(isira_handle h) { return h->cl_d; }
+
+// Counters of the inner solve in flight, once the stream has been synchronised.
+void finish_inner(isira_handle h) {
+    if (!h->pending_inner_stats) return;
+    const int its = hst(h)->inner_iters;
+    h->stats.inner_iters += its;
+    h->stats.spmv_launches += its;
+    if (h->pending_inner_stats > 0)
+        h->stats.kernel_launches += (long long)(h->pending_inner_stats > 1 ? h->pending_inner_stats : 3) * its;
+    else if (h->profiling) {
+        h->stats.inner_phase1_ms += 1e-6 * (double)hst(h)->prof_ns[0];
+        h->stats.inner_rows_ms += 1e-6 * (double)hst(h)->prof_ns[1];
+        h->stats.inner_phase2_ms += 1e-6 * (double)hst(h)->prof_ns[2];
+        h->stats.inner_phase1_timed += its;
+        h->stats.inner_phase1_csum += (long long)its * h->pending_c;
+    }
+    h->pending_inner_stats = 0;
+}
+
 // One inner solve on R (right-hand side) into Z (FP64, back-mapped).  Chunked mode returns the
-// iteration count; graph mode returns -1 (the count is read at the next synchronisation).
+// iteration count; graph mode and the one-launch solve return -1 (the count is read by finish_inner
+// after the next synchronisation).
 template <typename T>
 int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* Vt, int64_t ldv, double tau,
                  int max_it, bool gram_dirty, const double* R, const double* rnorm_dev, bool allow_graph,
@@ -291,6 +316,15 @@ int run_inner(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* 
     if (gram_dirty && c > 0) {
         gram_setup<T>(a, h->Gm, h->Cinv, h->partial, s);
         h->stats.kernel_launches += 1;
+    }
+    const ClusterPlan& plan = cluster_of<T>(h);
+    if (plan.ctas > 0 && h->opts.inner_graph) {
+        ck(cluster_minres<T>(a, plan, R, rnorm_dev, h->Z, h->profiling != 0, s));
+        h->stats.kernel_launches += 1;
+        h->stats.inner_solves += 1;
+        h->pending_inner_stats = -1;
+        h->pending_c = c;
+        return -1;
     }
     inner_prep_launch<T>(a, R, rnorm_dev, s);
     inner_phase2<T>(a, 1, s);
@@ -576,13 +610,7 @@ bool expand_basis(isira_handle h, int k, int c) {
         outer_cgs2(oa, k, c, s);
         h->stats.kernel_launches += 3;
         sync(h);
-        if (h->pending_inner_stats) {   // the graph-driven inner solve has finished by now
-            const int its = hst(h)->inner_iters;
-            h->stats.inner_iters += its;
-            h->stats.spmv_launches += its;
-            h->stats.kernel_launches += (long long)(h->pending_inner_stats > 1 ? h->pending_inner_stats : 3) * its;
-            h->pending_inner_stats = 0;
-        }
+        finish_inner(h);                // the inner solve has finished by now
         const double zin = hst(h)->cgs_in, zout = hst(h)->cgs_out;
         if (zout > 1e-10 * zin && zout > 0.0 && std::isfinite(zout)) {
             outer_expand(oa, k, h->lanes, s);
@@ -1065,6 +1093,11 @@ isira_status isira_create_weighted(isira_handle* out, int64_t n, int64_t nnz, co
         std::memset(h->hs, 0, sizeof(HostStatus));
         ck(cudaHostGetDevicePointer((void**)&h->hs_dev, h->hs, 0));
         h->rs.err = &h->hs_dev->dev_error;
+        {
+            unsigned long long* scr = reinterpret_cast<unsigned long long*>(h->dscratch);
+            cluster_plan<float>(rs, h->sell_total, scr, s, &h->cl_f);
+            cluster_plan<double>(rs, h->sell_total, scr, s, &h->cl_d);
+        }
         if (h->opts.precision == ISIRA_MIXED) alloc_inner(h, h->fb); else alloc_inner(h, h->db);
         if (h->opts.precond < -1 || h->opts.precond > 1) throw StatusError{ISIRA_ERR_INVALID_ARG};
         int chunk = h->opts.inner_chunk > 0 ? h->opts.inner_chunk : 16;
@@ -1408,6 +1441,8 @@ isira_status isira_inner_solve(isira_handle h, int precision, double sigma, int 
             sync(h);
             if (Vt) cudaFree(Vt);
         }
+        if (its < 0) its = hst(h)->inner_iters;
+        finish_inner(h);
         // back-map (Eq. 2.5): remove the mean; the trimmed entry is already zero
         OuterArgs oa = make_outer(h);
         outer_cgs2(oa, 0, 0, s);   // with an empty basis the two passes only subtract the mean
