@@ -449,9 +449,10 @@ __global__ void __launch_bounds__(kThreads) k_phase2(InnerArgs<T> a, int init, c
 
 // ------------------------------------------------------------------ stand-alone operator apply
 // y_r = (deg_r - sigma) x_r - g_r + (sigma/n) 1^T x + delta (Vh (Vh^T x))_r for r != trim, y_trim = 0, with
-// x in z0, its gathered sums in gsum and 1^T x, delta Vh^T x left in s_cur, u1 by k_opstats.
+// x in z0, its gathered sums in gsum and 1^T x, delta Vh^T x left in s_cur, u1 by k_opstats.  y goes
+// straight to the caller's vector and numbering (perm, null: the caller's is the solver's).
 template <typename T, int NC>
-__global__ void __launch_bounds__(kThreads) k_apply_rows(InnerArgs<T> a) {
+__global__ void __launch_bounds__(kThreads) k_apply_rows(InnerArgs<T> a, const int32_t* __restrict__ perm, T* yext) {
     constexpr int VN = Vec<T>::N;
     constexpr int NE = Ncols<NC>::value;
     const InnerState<T>* st = a.st;
@@ -464,7 +465,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_rows(InnerArgs<T> a) {
     const int64_t n = a.rs.n, trim = a.trim;
     const int64_t step = (int64_t)gridDim.x * blockDim.x * VN;
     for (int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * VN; r0 < n; r0 += step) {
-        T g[VN], z[VN], y[VN], vd[VN];
+        T g[VN], z[VN], vd[VN];
         T dgv[VN];
         vld(a.gsum + r0, g);
         vld(a.z0 + r0, z);
@@ -485,10 +486,42 @@ __global__ void __launch_bounds__(kThreads) k_apply_rows(InnerArgs<T> a) {
             const int64_t r = r0 + e;
             const T degT = dgv[e];
             const T v = ((degT - sigma) * z[e] - g[e] + s_term) + vd[e];
-            y[e] = (r < n && r != trim) ? v : T(0);
+            if (r < n) yext[perm ? perm[r] : r] = r != trim ? v : T(0);
         }
-        vst(a.Y + r0, y);
     }
+}
+
+// The same for graphs whose rows are all sliced, with the gather: one kernel, no neighbour sums stored.
+template <typename T>
+struct ApplyStore {
+    const InnerArgs<T>& a;
+    const T* u1s;
+    T sigma, s_term;
+    int c;
+    const int32_t* __restrict__ perm;
+    T* yext;
+    __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) {
+        T v = T(0);
+        if (r != a.trim) {
+            const T* dw = a.rs.template degw<T>();
+            const T degT = dw ? dw[r] : (T)a.deg[r];
+            T vd = T(0);
+            for (int t = 0; t < c; ++t) vd += a.Vt[(int64_t)t * a.ldv + r] * u1s[t];
+            v = ((degT - sigma) * a.z0[r] - s + s_term) + vd;
+        }
+        yext[perm ? perm[r] : r] = v;
+    }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 4) k_apply_slices(InnerArgs<T> a, const int32_t* __restrict__ perm, T* yext) {
+    __shared__ T u1s[kCMax];
+    const InnerState<T>* st = a.st;
+    const int c = st->p_c;
+    for (int t = threadIdx.x; t < c; t += blockDim.x) u1s[t] = st->u1[t];
+    __syncthreads();
+    ApplyStore<T> epi{a, u1s, st->p_sigma, st->p_sig_n * st->s_cur, c, perm, yext};
+    slices_only_gather<T>(a.rs, a.z0, epi, a.trim);
 }
 
 // ------------------------------------------------------------------ prep: b = rh / ||r||, h1 = Vh^T D^{-1} b
@@ -571,8 +604,11 @@ __global__ void __launch_bounds__(kThreads) k_finalize(InnerArgs<T> a, double* Z
 
 // ------------------------------------------------------------------ operator statistics for a stand-alone apply
 
+// Takes the caller's x and V (FP64, ld n, the caller's numbering) into z0 (trimmed entry 0) and Vt (a.Vt's
+// buffer, precision T), and forms 1^T x and Vh^T x on the way.
 template <typename T, int NC>
-__global__ void __launch_bounds__(kThreads) k_opstats(InnerArgs<T> a, const T* x) {
+__global__ void __launch_bounds__(kThreads) k_opstats(InnerArgs<T> a, const T* x, const double* V,
+                                                      const int32_t* __restrict__ perm, T* Vt) {
     __shared__ T red[1 + NC];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.st->p_sigma = a.sigma;
@@ -584,12 +620,18 @@ __global__ void __launch_bounds__(kThreads) k_opstats(InnerArgs<T> a, const T* x
     for (int t = 0; t < 1 + NC; ++t) acc[t] = T(0);
     const int64_t n = a.rs.n;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-        if (r == a.trim) continue;
-        const T xr = x[r];
+        const int64_t i = perm ? perm[r] : r;
+        const bool ok = r != a.trim;
+        const T xr = ok ? x[i] : T(0);
+        a.z0[r] = xr;
         acc[0] += xr;
 #pragma unroll
         for (int t = 0; t < NC; ++t)
-            if (t < a.c) acc[1 + t] += a.Vt[(int64_t)t * a.ldv + r] * xr;
+            if (t < a.c) {
+                const T v = (T)V[(int64_t)t * n + i];
+                Vt[(int64_t)t * a.ldv + r] = v;
+                if (ok) acc[1 + t] += v * xr;
+            }
     }
     if (block_partials_arrive<T, 1 + NC>(acc, 1 + a.c, a.partial, a.pstride, a.counter)) {
         last_block_sum(a.partial, a.pstride, gridDim.x, 1 + a.c, red, a.counter);
@@ -717,6 +759,19 @@ __global__ void __launch_bounds__(kThreads) k_gram(InnerArgs<T> a, double* G, do
             }
             for (int p = 0; p < c; ++p) Cinv[p + col * c] = y[p];
         }
+    }
+}
+
+// the caller's right-hand side and deflation vectors into the solver's numbering, V in precision T
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_stage_inputs(const double* __restrict__ r_in, const double* __restrict__ V,
+                                                           const int32_t* __restrict__ perm, int64_t n, int64_t ld,
+                                                           int c, double* __restrict__ R, T* __restrict__ Vt) {
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = perm ? perm[r] : r;
+        R[r] = r_in[i];
+#pragma unroll 4
+        for (int t = 0; t < c; ++t) Vt[(int64_t)t * ld + r] = (T)V[(int64_t)t * n + i];
     }
 }
 
@@ -1271,9 +1326,13 @@ void inner_phase1(const InnerArgs<T>& a, int lanes, cudaStream_t s) {
 }
 
 template <typename T>
-void inner_apply(const InnerArgs<T>& a, int lanes, cudaStream_t s) {
+void inner_apply(const InnerArgs<T>& a, int lanes, const int32_t* perm, T* y, cudaStream_t s) {
+    if (slices_only(a.rs)) {
+        k_apply_slices<T><<<slice_grid(a.rs), kThreads, 0, s>>>(a, perm, y);
+        return;
+    }
     inner_gather<T>(a, lanes, s);
-#define LA(NC) k_apply_rows<T, NC><<<wave_grid((const void*)k_apply_rows<T, NC>, vec_blocks(a)), kThreads, 0, s>>>(a)
+#define LA(NC) k_apply_rows<T, NC><<<wave_grid((const void*)k_apply_rows<T, NC>, vec_blocks(a)), kThreads, 0, s>>>(a, perm, y)
     ISIRA_NC_DISPATCH(a.c, LA);
 #undef LA
 }
@@ -1359,10 +1418,17 @@ void inner_finalize_to(const InnerArgs<T>& a, double* Z, cudaStream_t s) {
 }
 
 template <typename T>
-void inner_opstats(const InnerArgs<T>& a, const T* x, cudaStream_t s) {
-#define LS(NC) k_opstats<T, NC><<<wave_grid((const void*)k_opstats<T, NC>, a.ew_blocks), kThreads, 0, s>>>(a, x)
+void inner_opstats(const InnerArgs<T>& a, const T* x, const double* V, const int32_t* perm, T* Vt, cudaStream_t s) {
+#define LS(NC)                                                                                                  \
+    k_opstats<T, NC><<<wave_grid((const void*)k_opstats<T, NC>, a.ew_blocks), kThreads, 0, s>>>(a, x, V, perm, Vt)
     ISIRA_NC_DISPATCH(a.c, LS);
 #undef LS
+}
+
+template <typename T>
+void stage_inputs(const double* r_in, const double* V, const int32_t* perm, int64_t n, int64_t ld, int c, double* R,
+                  T* Vt, int blocks, cudaStream_t s) {
+    k_stage_inputs<T><<<blocks, kThreads, 0, s>>>(r_in, V, perm, n, ld, c, R, Vt);
 }
 
 template <typename T>
@@ -1384,7 +1450,7 @@ void copy_vcol(const double* src, T* dst, int64_t n, cudaStream_t s) {
 
 #define ISIRA_INSTANTIATE_INNER(T)                                                                        \
     template void inner_phase1<T>(const InnerArgs<T>&, int, cudaStream_t);                               \
-    template void inner_apply<T>(const InnerArgs<T>&, int, cudaStream_t);                                \
+    template void inner_apply<T>(const InnerArgs<T>&, int, const int32_t*, T*, cudaStream_t);            \
     template void inner_gather_vec<T>(const InnerArgs<T>&, const T*, T*, int, const int*, cudaStream_t);   \
     template void ml_inner_prep<T>(const InnerArgs<T>&, const double*, const double*, cudaStream_t);      \
     template void ml_phase1<T>(const InnerArgs<T>&, cudaStream_t);                                       \
@@ -1398,7 +1464,9 @@ void copy_vcol(const double* src, T* dst, int64_t n, cudaStream_t s) {
     template void inner_phase2_cond<T>(const InnerArgs<T>&, cudaGraphConditionalHandle, cudaStream_t);   \
     template void inner_prep_launch<T>(const InnerArgs<T>&, const double*, const double*, cudaStream_t); \
     template void inner_finalize_to<T>(const InnerArgs<T>&, double*, cudaStream_t);                      \
-    template void inner_opstats<T>(const InnerArgs<T>&, const T*, cudaStream_t);                         \
+    template void inner_opstats<T>(const InnerArgs<T>&, const T*, const double*, const int32_t*, T*, cudaStream_t); \
+    template void stage_inputs<T>(const double*, const double*, const int32_t*, int64_t, int64_t, int, double*, T*, \
+                                  int, cudaStream_t);                                                     \
     template void gram_setup<T>(const InnerArgs<T>&, double*, double*, double*, cudaStream_t);           \
     template void copy_vcol<T>(const double*, T*, int64_t, cudaStream_t);                                 \
     template cudaError_t inner_gather_attrs<T>(int);

@@ -120,8 +120,8 @@ template <typename T> void inner_prep_launch(const InnerArgs<T>& a, const double
                                              cudaStream_t s);
 template <typename T> void inner_phase1(const InnerArgs<T>& a, int lanes, cudaStream_t s);   // gather + rows
 template <typename T> void inner_gather(const InnerArgs<T>& a, int lanes, cudaStream_t s);
-// stand-alone operator apply: gather of z0, then Y = operator(z0) (after inner_opstats on z0)
-template <typename T> void inner_apply(const InnerArgs<T>& a, int lanes, cudaStream_t s);
+// stand-alone operator apply: y (the caller's vector and numbering) = operator(z0), after inner_opstats
+template <typename T> void inner_apply(const InnerArgs<T>& a, int lanes, const int32_t* perm, T* y, cudaStream_t s);
 // every gather kernel of precision T may take up to `bytes` of dynamic shared memory
 template <typename T> cudaError_t inner_gather_attrs(int bytes);
 template <typename T> void inner_rows(const InnerArgs<T>& a, cudaStream_t s);
@@ -130,7 +130,12 @@ template <typename T> void inner_phase2(const InnerArgs<T>& a, int init, cudaStr
 template <typename T> void inner_phase2_cond(const InnerArgs<T>& a, cudaGraphConditionalHandle cond,
                                              cudaStream_t s);
 template <typename T> void inner_finalize_to(const InnerArgs<T>& a, double* Z, cudaStream_t s);
-template <typename T> void inner_opstats(const InnerArgs<T>& a, const T* x, cudaStream_t s);
+// x, V: the caller's (perm null: in the solver's numbering); z0 and Vt receive the solver's copies
+template <typename T>
+void inner_opstats(const InnerArgs<T>& a, const T* x, const double* V, const int32_t* perm, T* Vt, cudaStream_t s);
+template <typename T>
+void stage_inputs(const double* r_in, const double* V, const int32_t* perm, int64_t n, int64_t ld, int c, double* R,
+                  T* Vt, int blocks, cudaStream_t s);
 template <typename T> void gram_setup(const InnerArgs<T>& a, double* G_out, double* Cinv_out, double* scratch,
                                       cudaStream_t s);
 template <typename T> void copy_vcol(const double* src, T* dst, int64_t n, cudaStream_t s);

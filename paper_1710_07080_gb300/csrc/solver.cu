@@ -109,6 +109,8 @@ struct isira_handle_s {
     double* R = nullptr;
     double* Z = nullptr;
     double* dscratch = nullptr;
+    void* vbuf = nullptr;         // component calls: the solver's copy of the caller's deflation vectors
+    size_t vbuf_bytes = 0;
     ArrowWork* arrow = nullptr;   // scratch of the warm-start Rayleigh-Ritz path
     double* gsum = nullptr;       // gather output, n doubles (shared by both precisions)
     double* partial = nullptr;
@@ -145,6 +147,9 @@ struct isira_handle_s {
 };
 
 namespace {
+
+// slot of dscratch that holds 1.0: the norm by which a right-hand side that is not scaled is divided
+constexpr int kOneSlot = 511;
 
 template <typename T>
 void alloc_inner(isira_handle h, InnerBuffers<T>& b) {
@@ -537,7 +542,7 @@ float time_inner(isira_handle h, InnerBuffers<T>& b, cudaEvent_t e0, cudaEvent_t
     const double tau = h->opts.tau_inner > 0.0 ? h->opts.tau_inner : 1e-3;
     const int max_it = h->opts.max_inner > 0 ? h->opts.max_inner : 5000;
     ck(cudaEventRecord(e0, s));
-    run_inner<T>(h, b, 0.0, 0, nullptr, h->ld, tau, max_it, false, h->R, h->dscratch + 300, true);
+    run_inner<T>(h, b, 0.0, 0, nullptr, h->ld, tau, max_it, false, h->R, h->dscratch + kOneSlot, true);
     ck(cudaEventRecord(e1, s));
     sync(h);
     float ms = 0.f;
@@ -562,8 +567,6 @@ void choose_preconditioner(isira_handle h) {
     OuterArgs oa = make_outer(h);
     outer_random(oa, h->opts.seed, 7777, h->stream);            // right-hand side in Z, copied to R
     ck(cudaMemcpyAsync(h->R, h->Z, sizeof(double) * (size_t)h->n, cudaMemcpyDeviceToDevice, h->stream));
-    const double one = 1.0;
-    ck(cudaMemcpyAsync(h->dscratch + 300, &one, sizeof(double), cudaMemcpyHostToDevice, h->stream));
     cudaEvent_t e0, e1;
     ck(cudaEventCreate(&e0));
     ck(cudaEventCreate(&e1));
@@ -661,7 +664,7 @@ template <typename T>
 float time_gather(isira_handle h, InnerBuffers<T>& b, int lanes, cudaEvent_t e0, cudaEvent_t e1) {
     cudaStream_t s = h->stream;
     InnerArgs<T> a = make_args<T>(h, b, 0.0, 0, nullptr, h->ld, 1e-3, 1);
-    inner_opstats<T>(a, a.z0, s);          // a fresh state: not done, iteration 0
+    inner_opstats<T>(a, a.z0, nullptr, nullptr, nullptr, s);   // a fresh state: not done, iteration 0
     float tot = 0.f;
     for (int rep = 0; rep < 4; ++rep) {
         ck(cudaEventRecord(e0, s));
@@ -752,7 +755,7 @@ void autotune_gather(isira_handle h) {
 
 void free_handle(isira_handle h) {
     if (!h) return;
-    void* ptrs[] = {h->own_w, h->wf, h->degwd, h->degwf, h->sell_wd, h->sell_wf, h->gsum, h->deg32, h->sell_off, h->sell_ci, h->own_rp, h->own_ci, h->perm, h->inv, h->item_row, h->item_k, h->item_partial,
+    void* ptrs[] = {h->vbuf, h->own_w, h->wf, h->degwd, h->degwf, h->sell_wd, h->sell_wf, h->gsum, h->deg32, h->sell_off, h->sell_ci, h->own_rp, h->own_ci, h->perm, h->inv, h->item_row, h->item_k, h->item_partial,
                     h->item_count, h->warp_start, h->U, h->W, h->V, h->H, h->theta, h->S, h->R, h->Z, h->dscratch,
                     h->arrow, h->partial, h->counter, h->Gm, h->Cinv, h->lam_dev, h->tres_dev, h->fb.base, h->fb.st,
                     h->db.base, h->db.st, h->Vt_f, h->fb.ml, h->db.ml, h->ml_dv};
@@ -780,24 +783,31 @@ isira_status map_cuda(cudaError_t e) {
 
 namespace {
 
-// V (caller's numbering, n-by-c, ld n) into the solver's numbering, ld h->ld, precision T
+// Buffer for the solver's copy of a component call's deflation vectors (c columns of precision T, ld
+// h->ld).  The handle keeps it between calls up to kKeepV bytes: allocating and freeing it on each
+// call cost more than a small operator application (both synchronise the device).
+constexpr size_t kKeepV = (size_t)1 << 30;
+
 template <typename T>
-T* internal_V(isira_handle h, const double* d_V, int c, cudaStream_t s) {
+T* v_buffer(isira_handle h, int c) {
     if (c <= 0) return nullptr;
-    double* Vd = nullptr;
-    ck(cudaMalloc(&Vd, sizeof(double) * (size_t)h->ld * c));
-    for (int t = 0; t < c; ++t) {
-        if (h->perm) to_internal<double>(d_V + (size_t)t * h->n, h->perm, h->n, Vd + (size_t)t * h->ld, s);
-        else ck(cudaMemcpyAsync(Vd + (size_t)t * h->ld, d_V + (size_t)t * h->n, sizeof(double) * h->n,
-                                cudaMemcpyDeviceToDevice, s));
+    const size_t bytes = sizeof(T) * (size_t)h->ld * c;
+    if (bytes > h->vbuf_bytes) {
+        if (h->vbuf) cudaFree(h->vbuf);
+        h->vbuf = nullptr;
+        h->vbuf_bytes = 0;
+        ck(cudaMalloc(&h->vbuf, bytes));
+        h->vbuf_bytes = bytes;
     }
-    if (sizeof(T) == sizeof(double)) return reinterpret_cast<T*>(Vd);
-    float* Vf = nullptr;
-    ck(cudaMalloc(&Vf, sizeof(float) * (size_t)h->ld * c));
-    for (int t = 0; t < c; ++t) copy_vcol<float>(Vd + (size_t)t * h->ld, Vf + (size_t)t * h->ld, h->n, s);
-    ck(cudaStreamSynchronize(s));
-    cudaFree(Vd);
-    return reinterpret_cast<T*>(Vf);
+    return static_cast<T*>(h->vbuf);
+}
+
+// after the call has been synchronised
+void v_buffer_done(isira_handle h) {
+    if (h->vbuf_bytes <= kKeepV) return;
+    cudaFree(h->vbuf);
+    h->vbuf = nullptr;
+    h->vbuf_bytes = 0;
 }
 
 template <typename T>
@@ -805,17 +815,12 @@ void apply_operator_t(isira_handle h, InnerBuffers<T>& b, double sigma, int c, c
                       T* d_y) {
     cudaStream_t s = h->stream;
     alloc_inner(h, b);
-    T* Vt = internal_V<T>(h, d_V, c, s);
+    T* Vt = v_buffer<T>(h, c);
     InnerArgs<T> a = make_args<T>(h, b, sigma, c, Vt, h->ld, 1e-3, 1);
-    if (h->perm) to_internal<T>(d_x, h->perm, h->n, a.z0, s);
-    else ck(cudaMemcpyAsync(a.z0, d_x, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
-    ck(cudaMemsetAsync(a.z0 + h->trim, 0, sizeof(T), s));   // x_i is treated as 0
-    inner_opstats<T>(a, a.z0, s);
-    inner_apply<T>(a, h->lanes, s);
-    if (h->perm) to_external<T>(a.Y, h->perm, h->n, d_y, s);
-    else ck(cudaMemcpyAsync(d_y, a.Y, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
+    inner_opstats<T>(a, d_x, d_V, h->perm, Vt, s);
+    inner_apply<T>(a, h->lanes, h->perm, d_y, s);
     sync(h);
-    if (Vt) cudaFree(Vt);
+    v_buffer_done(h);
 }
 
 }  // namespace
@@ -1085,6 +1090,8 @@ isira_status isira_create_weighted(isira_handle* out, int64_t n, int64_t nnz, co
         ck(cudaMalloc(&h->deg32, sizeof(int32_t) * (size_t)h->ld));
         setup_deg32(d_row_ptr, n, h->ld, h->deg32, s);
         ck(cudaMalloc(&h->dscratch, sizeof(double) * 512));
+        const double one = 1.0;
+        ck(cudaMemcpyAsync(h->dscratch + kOneSlot, &one, sizeof(double), cudaMemcpyHostToDevice, s));
         ck(cudaMalloc(&h->Gm, sizeof(double) * kCMax * kCMax));
         ck(cudaMalloc(&h->Cinv, sizeof(double) * kCMax * kCMax));
         ck(cudaMalloc(&h->lam_dev, sizeof(double) * kCMax));
@@ -1423,24 +1430,21 @@ isira_status isira_inner_solve(isira_handle h, int precision, double sigma, int 
     try {
         cudaStream_t s = h->stream;
         // the right-hand side goes through the residual buffer, its norm through the scalar area
-        if (h->perm) to_internal<double>(d_r, h->perm, h->n, h->R, s);
-        else ck(cudaMemcpyAsync(h->R, d_r, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, s));
-        const double one = 1.0;
-        ck(cudaMemcpyAsync(h->dscratch + 300, &one, sizeof(double), cudaMemcpyHostToDevice, s));
+        const double* rnorm = h->dscratch + kOneSlot;
         int its = 0;
         if (precision == ISIRA_MIXED) {
             alloc_inner(h, h->fb);
-            float* Vt = internal_V<float>(h, d_V, c, s);
-            its = run_inner<float>(h, h->fb, sigma, c, Vt, h->ld, tau, max_it, true, h->R, h->dscratch + 300);
-            sync(h);
-            if (Vt) cudaFree(Vt);
+            float* Vt = v_buffer<float>(h, c);
+            stage_inputs<float>(d_r, d_V, h->perm, h->n, h->ld, c, h->R, Vt, h->ew_blocks, s);
+            its = run_inner<float>(h, h->fb, sigma, c, Vt, h->ld, tau, max_it, true, h->R, rnorm);
         } else {
             alloc_inner(h, h->db);
-            double* Vt = internal_V<double>(h, d_V, c, s);
-            its = run_inner<double>(h, h->db, sigma, c, Vt, h->ld, tau, max_it, true, h->R, h->dscratch + 300);
-            sync(h);
-            if (Vt) cudaFree(Vt);
+            double* Vt = v_buffer<double>(h, c);
+            stage_inputs<double>(d_r, d_V, h->perm, h->n, h->ld, c, h->R, Vt, h->ew_blocks, s);
+            its = run_inner<double>(h, h->db, sigma, c, Vt, h->ld, tau, max_it, true, h->R, rnorm);
         }
+        sync(h);
+        v_buffer_done(h);
         if (its < 0) its = hst(h)->inner_iters;
         finish_inner(h);
         // back-map (Eq. 2.5): remove the mean; the trimmed entry is already zero
