@@ -19,6 +19,7 @@
 // Vectors per row and iteration: z_k (gathered), z_{k-1}, Y, three rotating w
 // buffers, x, and c columns of Vh.
 #pragma once
+#include <algorithm>
 #include <mutex>
 #include <unordered_map>
 
@@ -654,20 +655,30 @@ __global__ void __launch_bounds__(kThreads) k_opstats(InnerArgs<T> a, const T* x
 // ------------------------------------------------------------------ Gram matrix Vh^T D^{-1} Vh and C^{-1}
 
 constexpr int kGramTile = 128;
+constexpr int kGramBlocks = 456;        // three CTAs per SM: the last CTA adds one partial per CTA and entry
 
+// G = Vh^T D^{-1} Vh over the untrimmed rows, and C^{-1} = (delta^{-1} I + G)^{-1}.  A tile of scaled rows sits in
+// shared memory; the c (c + 1) / 2 entries are dealt to the threads, several row segments to an entry
+// while there are threads left (c = 4: 25 segments of 10 entries; one thread per entry, as before, left 246 of 256
+// idle and the Cholesky factorisation and the inverse to a single one).  The last CTA factors C with
+// one lane per row and inverts it with one lane per column.  Bound by the FP64 pipe: n c^2 / 2 FMAs.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_gram(InnerArgs<T> a, double* G, double* Cinv, double* partial,
                                                    int pstride) {
     extern __shared__ double gsm[];     // [c][kGramTile + 1]
-    const int c = a.c;
+    __shared__ double rs[kGramTile];
+    __shared__ double red[2 * kThreads];
+    const int c = a.c, tid = threadIdx.x;
     const int ne = c * (c + 1) / 2;
     const int64_t n = a.rs.n;
     constexpr int kPer = 2;             // entries per thread (c <= 31 -> ne <= 496 <= 2 * 256)
+    const int nseg = ne <= kThreads ? kThreads / ne : 1;
+    const int seg = ne <= kThreads ? tid / ne : 0;
     int ea[kPer], eb[kPer];
     double acc[kPer];
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        int e = threadIdx.x + q * blockDim.x;
+        int e = ne <= kThreads ? (q == 0 && seg < nseg ? tid % ne : ne) : tid + q * kThreads;
         acc[q] = 0.0;
         ea[q] = -1;
         eb[q] = -1;
@@ -681,15 +692,17 @@ __global__ void __launch_bounds__(kThreads) k_gram(InnerArgs<T> a, double* G, do
     const int ldt = kGramTile + 1;
     for (int64_t r0 = (int64_t)blockIdx.x * kGramTile; r0 < n; r0 += (int64_t)gridDim.x * kGramTile) {
         __syncthreads();
-        for (int idx = threadIdx.x; idx < c * kGramTile; idx += blockDim.x) {
+        for (int rr = tid; rr < kGramTile; rr += kThreads) {
+            const int64_t r = r0 + rr;
+            double w = 0.0;
+            if (r < n && r != a.trim) w = rsqrt((double)precond_diag(row_degree<T>(a.rs, r), a.sigma));
+            rs[rr] = w;
+        }
+        __syncthreads();
+        for (int idx = tid; idx < c * kGramTile; idx += kThreads) {
             const int col = idx / kGramTile, rr = idx % kGramTile;
             const int64_t r = r0 + rr;
-            double v = 0.0;
-            if (r < n && r != a.trim) {
-                const T degT = row_degree<T>(a.rs, r);
-                v = (double)a.Vt[(int64_t)col * a.ldv + r] * rsqrt((double)precond_diag(degT, a.sigma));
-            }
-            gsm[col * ldt + rr] = v;
+            gsm[col * ldt + rr] = r < n && r != a.trim ? (double)a.Vt[(int64_t)col * a.ldv + r] * rs[rr] : 0.0;
         }
         __syncthreads();
 #pragma unroll
@@ -697,68 +710,75 @@ __global__ void __launch_bounds__(kThreads) k_gram(InnerArgs<T> a, double* G, do
             if (ea[q] >= 0) {
                 const double* pa = gsm + ea[q] * ldt;
                 const double* pb = gsm + eb[q] * ldt;
-                double s = 0.0;
-                for (int rr = 0; rr < kGramTile; ++rr) s += pa[rr] * pb[rr];
-                acc[q] += s;
+                double s0 = 0.0, s1 = 0.0;
+                int rr = seg;
+                for (; rr + nseg < kGramTile; rr += 2 * nseg) {
+                    s0 += pa[rr] * pb[rr];
+                    s1 += pa[rr + nseg] * pb[rr + nseg];
+                }
+                if (rr < kGramTile) s0 += pa[rr] * pb[rr];
+                acc[q] += s0 + s1;
             }
         }
     }
     // per-block partials (one slot per entry), then the last block sums and factors
-    for (int q = 0; q < kPer; ++q) {
-        int e = threadIdx.x + q * blockDim.x;
-        if (e < ne) partial[(size_t)e * pstride + blockIdx.x] = acc[q];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) red[tid + q * kThreads] = acc[q];
+    __syncthreads();
+    for (int e = tid; e < ne; e += kThreads) {
+        double s = red[e];
+        for (int g = 1; g < nseg; ++g) s += red[e + g * ne];
+        partial[(size_t)e * pstride + blockIdx.x] = s;
     }
     __threadfence();
     __syncthreads();
     __shared__ int last;
-    if (threadIdx.x == 0) last = (atomicAdd(a.counter, 1u) == gridDim.x - 1);
+    if (tid == 0) last = (atomicAdd(a.counter, 1u) == gridDim.x - 1);
     __syncthreads();
     if (!last) return;
-    __shared__ double Gs[kCMax * kCMax];
-    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < (int)gridDim.x; ++b) s += __ldcg(partial + (size_t)e * pstride + b);
+    last_block_sum(partial, pstride, gridDim.x, ne, red, a.counter);
+    constexpr int L = kCMax + 1;
+    __shared__ double A[kCMax * L], Y[kCMax * L];
+    const double dinv = 1.0 / (double)a.delta;
+    for (int e = tid; e < ne; e += kThreads) {
+        const double s = red[e];
         int p = 0, rem = e;
         while (rem >= c - p) { rem -= c - p; ++p; }
-        Gs[p + (p + rem) * c] = s;
-        Gs[(p + rem) + p * c] = s;
+        const int q = p + rem;
+        G[p + q * c] = s;
+        G[q + p * c] = s;
+        A[q * L + p] = p == q ? s + dinv : s;              // lower triangle of C
     }
-    if (threadIdx.x == 0) *a.counter = 0u;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        // C = delta^{-1} I + G (SPD), Cholesky C = L L^T, then C^{-1} column by column
-        double Lc[kCMax * kCMax];
-        const double dinv = 1.0 / (double)a.delta;
-        for (int p = 0; p < c; ++p)
-            for (int s = 0; s < c; ++s) {
-                G[p + s * c] = Gs[p + s * c];
-                Lc[p + s * c] = 0.0;
-            }
-        for (int s = 0; s < c; ++s) {
-            double d = Gs[s + s * c] + dinv;
-            for (int t = 0; t < s; ++t) d -= Lc[s + t * c] * Lc[s + t * c];
-            d = sqrt(d > 0.0 ? d : 1e-300);
-            Lc[s + s * c] = d;
-            for (int p = s + 1; p < c; ++p) {
-                double v = Gs[p + s * c];
-                for (int t = 0; t < s; ++t) v -= Lc[p + t * c] * Lc[s + t * c];
-                Lc[p + s * c] = v / d;
-            }
+    if (tid >= 32) return;
+    // C = delta^{-1} I + G (SPD), Cholesky C = L L^T in place, then C^{-1} column by column
+    const int lane = tid;
+    for (int s = 0; s < c; ++s) {
+        if (lane == s) {
+            const double d = A[s * L + s];
+            A[s * L + s] = sqrt(d > 0.0 ? d : 1e-300);
         }
-        for (int col = 0; col < c; ++col) {
-            double y[kCMax];
-            for (int p = 0; p < c; ++p) {
-                double v = (p == col) ? 1.0 : 0.0;
-                for (int t = 0; t < p; ++t) v -= Lc[p + t * c] * y[t];
-                y[p] = v / Lc[p + p * c];
-            }
-            for (int p = c - 1; p >= 0; --p) {
-                double v = y[p];
-                for (int t = p + 1; t < c; ++t) v -= Lc[t + p * c] * y[t];
-                y[p] = v / Lc[p + p * c];
-            }
-            for (int p = 0; p < c; ++p) Cinv[p + col * c] = y[p];
+        __syncwarp();
+        if (lane > s && lane < c) A[lane * L + s] /= A[s * L + s];
+        __syncwarp();
+        if (lane > s && lane < c) {
+            const double l = A[lane * L + s];
+            for (int q = s + 1; q <= lane; ++q) A[lane * L + q] -= l * A[q * L + s];
         }
+        __syncwarp();
+    }
+    if (lane < c) {
+        for (int p = 0; p < c; ++p) {
+            double v = (p == lane) ? 1.0 : 0.0;
+            for (int t = lane; t < p; ++t) v -= A[p * L + t] * Y[t * L + lane];
+            Y[p * L + lane] = p < lane ? 0.0 : v / A[p * L + p];
+        }
+        for (int p = c - 1; p >= 0; --p) {
+            double v = Y[p * L + lane];
+            for (int t = p + 1; t < c; ++t) v -= A[t * L + p] * Y[t * L + lane];
+            Y[p * L + lane] = v / A[p * L + p];
+        }
+        for (int p = 0; p < c; ++p) Cinv[p + lane * c] = Y[p * L + lane];
     }
 }
 
@@ -1440,7 +1460,7 @@ void gram_setup(const InnerArgs<T>& a, double* G_out, double* Cinv_out, double* 
         cudaFuncSetAttribute(k_gram<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(sizeof(double) * kCMax * (kGramTile + 1)));
     });
-    k_gram<T><<<a.ew_blocks, kThreads, smem, s>>>(a, G_out, Cinv_out, partial, a.pstride);
+    k_gram<T><<<std::min(a.ew_blocks, kGramBlocks), kThreads, smem, s>>>(a, G_out, Cinv_out, partial, a.pstride);
 }
 
 template <typename T>

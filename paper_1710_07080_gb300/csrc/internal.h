@@ -219,6 +219,8 @@ void outer_arrow_eig(const double* H, int ldh, int k, int w, double* theta, doub
 // Z <- Z - Q(Q^T Z) - mean(Z) twice, then ||Z||, for Q = [U(:,0:k) V(:,0:c)]; Z already holds the
 // FP64 input.  Writes cgs_in / cgs_out to the host status.
 void outer_cgs2(const OuterArgs& a, int k, int c, cudaStream_t s);
+// out (the caller's vector and numbering) <- Z - mean(Z) 1
+void outer_center(const OuterArgs& a, const int32_t* perm, double* out, cudaStream_t s);
 // U(:,k) = Z/||Z||, W(:,k) = L U(:,k), H(0:k, k) = U(:,0:k+1)^T W(:,k) (and the symmetric row).
 void outer_expand(const OuterArgs& a, int k, int lanes, cudaStream_t s);
 cudaError_t outer_gather_attrs(int bytes);

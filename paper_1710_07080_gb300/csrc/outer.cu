@@ -914,6 +914,38 @@ void outer_cgs2(const OuterArgs& a, int k, int c, cudaStream_t s) {
         a, k, c, a.Z, a.Z, cB, nullptr, nullptr, 0);
 }
 
+// ------------------------------------------------------------------ back-map of a single inner solve
+// Z minus its mean, twice (the second pass removes what rounding left), to the caller's vector and
+// numbering.  These are the three passes that Gram-Schmidt with an empty basis would make, without its
+// staging: 3 x 3 us against 45 us at n = 12,339.
+
+// STEP 0: mean of Z;  STEP 1: Z -= mean, mean of the result;  STEP 2: out = Z - mean
+template <int STEP>
+__global__ void __launch_bounds__(kThreads) k_center(OuterArgs a, const double* mean, double* mean_next,
+                                                     const int32_t* __restrict__ perm, double* out) {
+    const double m = STEP == 0 ? 0.0 : *mean;
+    double acc[1] = {0.0};
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < a.n; r += (int64_t)gridDim.x * blockDim.x) {
+        const double z = STEP == 0 ? a.Z[r] : a.Z[r] - m;
+        if (STEP == 1) a.Z[r] = z;
+        if (STEP == 2) out[perm ? perm[r] : r] = z;
+        acc[0] += z;
+    }
+    if (STEP == 2) return;
+    __shared__ double red[1];
+    if (block_partials_arrive<double, 1>(acc, 1, a.partial, a.pstride, a.counter)) {
+        last_block_sum(a.partial, a.pstride, gridDim.x, 1, red, a.counter);
+        if (threadIdx.x == 0) *mean_next = red[0] / (double)a.n;
+    }
+}
+
+void outer_center(const OuterArgs& a, const int32_t* perm, double* out, cudaStream_t s) {
+    double* m = a.dscratch + 8;
+    k_center<0><<<a.ew_blocks, kThreads, 0, s>>>(a, nullptr, m, nullptr, nullptr);
+    k_center<1><<<a.ew_blocks, kThreads, 0, s>>>(a, m, m + 1, nullptr, nullptr);
+    k_center<2><<<a.ew_blocks, kThreads, 0, s>>>(a, m + 1, nullptr, perm, out);
+}
+
 // ------------------------------------------------------------------ expand
 
 // Plain gather g[r] = sum_{c in N(r)} x[c] over the full Laplacian (no trimmed row).

@@ -253,6 +253,36 @@ volatile HostStatus* hst(isira_handle h) { return h->hs; }
 
 int nc_bucket(int c) { return c == 0 ? 0 : (c <= 8 ? 1 : (c <= 12 ? 2 : (c <= 16 ? 3 : (c <= 24 ? 4 : 5)))); }
 
+// Iterations of one inner solve from the host, without waiting for the stream: the device writes its
+// iteration count and its stopping flag to mapped host memory, and the host keeps `ahead` iterations
+// enqueued beyond the count it sees, so at most that many run empty after the stop (a check after
+// chunks of 16 left 8 on average, of 3 or 16 launches each).  Ends with the stream synchronised.
+// Returns the number of iterations enqueued.
+template <typename F>
+int run_ahead(isira_handle h, int max_it, int ahead, F launch) {
+    volatile HostStatus* st = hst(h);
+    int launched = 0;
+    for (long long polls = 0; !st->inner_done && launched < max_it;) {
+        if (launched - st->inner_iters < ahead) {
+            launch();
+            ++launched;
+        } else if ((++polls & 0xfff) == 0) {
+            const cudaError_t e = cudaStreamQuery(h->stream);
+            if (e == cudaErrorNotReady) continue;
+            ck(e);
+            if (launched - st->inner_iters >= ahead && !st->inner_done) break;   // idle without progress
+        }
+    }
+    sync(h);
+    return launched;
+}
+
+// before the launches of a solve that run_ahead drives (the stream holds no earlier work of the handle)
+void reset_inner_status(isira_handle h) {
+    hst(h)->inner_done = 0;
+    hst(h)->inner_iters = 0;
+}
+
 // WHILE(cond) { phase 1; phase 2 } with phase 2's last CTA setting cond = !done.  The kernels
 // read the per-solve shift and rank from device state, so one graph serves every solve of a bucket.
 template <typename T>
@@ -331,9 +361,23 @@ int run_inner(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* 
         h->pending_c = c;
         return -1;
     }
+    const bool ahead = !allow_graph && h->opts.inner_graph && !h->profiling && !h->sync_ev;
+    if (ahead) reset_inner_status(h);
     inner_prep_launch<T>(a, R, rnorm_dev, s);
     inner_phase2<T>(a, 1, s);
     h->stats.kernel_launches += 2;
+    if (ahead) {
+        const int nl = run_ahead(h, max_it, 4, [&] {
+            inner_phase1<T>(a, h->lanes, s);
+            inner_phase2<T>(a, 0, s);
+        });
+        inner_finalize_to<T>(a, h->Z, s);
+        h->stats.spmv_launches += nl;
+        h->stats.kernel_launches += 3 * nl + 1;
+        h->stats.inner_solves += 1;
+        h->stats.inner_iters += hst(h)->inner_iters;
+        return hst(h)->inner_iters;
+    }
     if (allow_graph && h->opts.inner_graph && !h->profiling) {
         const int bkt = nc_bucket(c);
         if (!h->inner_graph[bkt]) h->inner_graph[bkt] = build_inner_graph<T>(h, a);
@@ -464,6 +508,8 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
         for (int t = 0; t < c; ++t) dv[t] = 1.0 / ((lam ? lam[t] : 0.0) - sigma + h->delta);
         ck(cudaMemcpyAsync(h->ml_dv, dv, sizeof(double) * c, cudaMemcpyHostToDevice, s));
     }
+    const bool ahead = !allow_graph && h->opts.inner_graph && !h->profiling && !h->sync_ev;
+    if (ahead) reset_inner_status(h);
     ml_inner_prep<T>(a, R, rnorm_dev, s);
     ml_phase2a<T>(a, 1, s);
     ml_project<T>(a, 1, s);
@@ -473,6 +519,15 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
     ml_phase2c<T>(a, 1, s);
     const int per_it = ml_launches_per_iteration(b, c);
     h->stats.kernel_launches += per_it - 1;
+    if (ahead) {
+        const int nl = run_ahead(h, max_it, 2, [&] { ml_iteration<T>(h, b, a, cudaGraphConditionalHandle{}, 0, s); });
+        inner_finalize_to<T>(a, h->Z, s);
+        h->stats.spmv_launches += nl;
+        h->stats.kernel_launches += (long long)per_it * nl + 1;
+        h->stats.inner_solves += 1;
+        h->stats.inner_iters += hst(h)->inner_iters;
+        return hst(h)->inner_iters;
+    }
     if (allow_graph && h->opts.inner_graph && !h->profiling) {
         const int bkt = nc_bucket(c);
         if (!h->ml_graph[bkt]) h->ml_graph[bkt] = build_ml_graph<T>(h, b, a);
@@ -1449,9 +1504,7 @@ isira_status isira_inner_solve(isira_handle h, int precision, double sigma, int 
         finish_inner(h);
         // back-map (Eq. 2.5): remove the mean; the trimmed entry is already zero
         OuterArgs oa = make_outer(h);
-        outer_cgs2(oa, 0, 0, s);   // with an empty basis the two passes only subtract the mean
-        if (h->perm) to_external<double>(h->Z, h->perm, h->n, d_z, s);
-        else ck(cudaMemcpyAsync(d_z, h->Z, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, s));
+        outer_center(oa, h->perm, d_z, s);
         sync(h);
         if (iters) *iters = its;
         if (relres) *relres = hst(h)->inner_relres;
