@@ -821,6 +821,33 @@ __global__ void k_copy_vcol(const double* src, T* dst, int64_t n) {
 //       beta_{k+1}^2 = r^T w + h^T tv, Givens step;
 //   ml_phase2c: z_{k+1} = w + Vh tv (= Pi w + Vh D h), 1^T z_{k+1} and g_{k+1} = Vh^T z_{k+1}.
 
+// end of phase 1: alpha' summed over the CTAs; the last CTA adds the deflation part
+template <typename T>
+__device__ __forceinline__ void ml_phase1_finish(const InnerArgs<T>& a, T acc0, int c, T beta) {
+    InnerState<T>* st = a.st;
+    __shared__ T red[1];
+    T accv[1] = {acc0};
+    if (block_partials_arrive<T, 1>(accv, 1, a.partial, a.pstride, a.counter)) {
+        last_block_sum(a.partial, a.pstride, gridDim.x, 1, red, a.counter);
+        if (threadIdx.x == 0) {
+            // g_k = Vh^T z_k was reduced by the phase-2c launch that wrote z_k
+            const double bt = (double)beta, delta = (double)a.delta;
+            double al = (double)red[0];
+            for (int t = 0; t < c; ++t) {
+                const double gn = (double)st->g_cur[t];
+                const double u = delta * gn / bt;
+                st->u1[t] = (T)u;
+                al += gn / bt * u;
+            }
+            st->alpha = (T)al;
+        }
+    }
+}
+
+// resident CTAs per SM of the kernels that do row arithmetic in a sliced gather: FP32 wants the warps in
+// flight; in FP64 every CTA's reduction costs FP64 issue slots (a warp sum as much as five rows)
+template <typename T> struct SlicedRows { static constexpr int ctas = sizeof(T) == 4 ? 6 : 4; };
+
 template <typename T, int NC>
 __global__ void __launch_bounds__(kThreads) k_ml_phase1(InnerArgs<T> a) {
     constexpr int VN = Vec<T>::N;
@@ -884,23 +911,67 @@ __global__ void __launch_bounds__(kThreads) k_ml_phase1(InnerArgs<T> a) {
             }
         }
     }
-    __shared__ T red[1];
-    T accv[1] = {acc0};
-    if (block_partials_arrive<T, 1>(accv, 1, a.partial, a.pstride, a.counter)) {
-        last_block_sum(a.partial, a.pstride, gridDim.x, 1, red, a.counter);
-        if (threadIdx.x == 0) {
-            // g_k = Vh^T z_k was reduced by the phase-2c launch that wrote z_k
-            const double bt = (double)beta, delta = (double)a.delta;
-            double al = (double)red[0];
-            for (int t = 0; t < c; ++t) {
-                const double gn = (double)st->g_cur[t];
-                const double u = delta * gn / bt;
-                st->u1[t] = (T)u;
-                al += gn / bt * u;
-            }
-            st->alpha = (T)al;
+    ml_phase1_finish<T>(a, acc0, c, beta);
+}
+
+// The same with the gather, for graphs whose rows are all sliced: a lane has its row's neighbour sum and
+// does the row at once, so the sums are neither stored nor read and a launch falls away (118 x 109 x 101
+// grid, FP32: 12 + 15.4 us as two kernels).
+template <typename T>
+struct MlPhase1Row {
+    const InnerArgs<T>& a;
+    const T* __restrict__ zc;
+    const T* __restrict__ zp;
+    const T* __restrict__ wo1;
+    const T* __restrict__ wo2;
+    T* __restrict__ wn;
+    const T* __restrict__ dw;
+    T sigma, s_term, inv_beta, inv_oldb, cprev, oldeps, dlt, inv_gamma, phi, acc;
+    bool has_prev;
+    __device__ __forceinline__ void operator()(int64_t r, int64_t, T g) {
+        const bool ok = r != a.trim;
+        const T z = zc[r];
+        const T deg = dw ? dw[r] : (T)a.deg[r];
+        T y = ((deg - sigma) * z - g + s_term) * inv_beta;
+        if (has_prev) {
+            y -= cprev * a.rprev[r];
+            const T w = (zp[r] * inv_oldb - oldeps * wo2[r] - dlt * wo1[r]) * inv_gamma;
+            wn[r] = ok ? w : T(0);
+            if (ok) a.x[r] += phi * w;
         }
+        y = ok ? y : T(0);
+        a.Y[r] = y;
+        acc += z * inv_beta * y;
     }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, SlicedRows<T>::ctas) k_ml_phase1_s(InnerArgs<T> a) {
+    InnerState<T>* st = a.st;
+    if (st->done) return;
+    const int k = st->itn + 1;
+    const T beta = st->beta, oldb = st->oldb;
+    const bool has_prev = k >= 2;
+    MlPhase1Row<T> row{a,
+                       ((k - 1) & 1) ? a.z1 : a.z0,
+                       (k & 1) ? a.z1 : a.z0,
+                       wbuf(a, k + 1),                       // w_{j-1}, w_{j-2}, w_j of iteration j = k - 1
+                       wbuf(a, k),
+                       wbuf(a, k - 1),
+                       a.rs.template degw<T>(),
+                       st->p_sigma,
+                       st->p_sig_n * st->s_cur,
+                       T(1) / beta,
+                       has_prev ? T(1) / oldb : T(0),
+                       has_prev ? beta / oldb : T(0),
+                       st->w_oldeps,
+                       st->w_dlt,
+                       st->w_inv_gamma,
+                       st->w_phi,
+                       T(0),
+                       has_prev};
+    slices_only_gather<T>(a.rs, row.zc, row, a.trim);
+    ml_phase1_finish<T>(a, row.acc, st->p_c, beta);
 }
 
 // r_{k+1} = y' + Vh u1 - (alpha_k / beta_k) r_k (rprev <- r_k, rcur <- r_{k+1}) and h = Vh^T r_{k+1};
@@ -956,6 +1027,13 @@ __global__ void __launch_bounds__(kThreads) k_ml_phase2a(InnerArgs<T> a, int ini
                 }
                 vst(a.rprev + r0, rc);
                 vst(a.rcur + r0, rn);
+            }
+            if (NE == 0 && a.ml_x0) {              // nothing to project: the V-cycle's x0 = w D^{-1} r
+                T di[VN];
+                vld(a.ml_dinv0 + r0, di);
+#pragma unroll
+                for (int e = 0; e < VN; ++e) di[e] = a.ml_omega * rn[e] * di[e];
+                vst(a.ml_x0 + r0, di);
             }
         }
         if (NE > 0 && c > 0) {
@@ -1103,6 +1181,60 @@ __global__ void __launch_bounds__(kThreads) k_ml_phase2b(InnerArgs<T> a, int ini
     }
 }
 
+// The V-cycle's last gather (W x1) with level 0's post-smoothing and phase 2b's sums, for graphs whose rows are
+// all sliced and c <= 8 (NC = 0 or 8; more columns want more registers than a gather can spare).
+// Without deflation z_{k+1} = w: it is stored at once and phase 2c falls away.
+template <typename T, int NC>
+struct MlPostRow {
+    static constexpr int NE = NC;
+    const InnerArgs<T>& a;
+    T* __restrict__ out;
+    int c;
+    T acc[2 + NE];                                     // r^T w, (c = 0) 1^T w, Vh^T w
+    __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) {
+        const bool ok = r != a.trim;
+        const T x1 = a.ml_x1[r], di = a.ml_dinv0[r], b = a.ml_b0[r];
+        T w = x1 + a.ml_omega * (b * di - x1 + s * di);
+        w = ok ? w : T(0);
+        out[r] = w;
+        acc[0] += (ok ? (NC == 0 ? b : a.rcur[r]) : T(0)) * w;
+        if (NC == 0) acc[1] += w;
+#pragma unroll
+        for (int t = 0; t < NE; ++t)
+            if (t < c && ok) acc[2 + t] += a.Vt[(int64_t)t * a.ldv + r] * w;
+    }
+};
+
+template <typename T, int NC>
+__global__ void __launch_bounds__(kThreads, SlicedRows<T>::ctas) k_ml_post_s(InnerArgs<T> a, int init,
+                                                                           cudaGraphConditionalHandle cond,
+                                                                           int has_cond) {
+    constexpr int NA = 2 + NC;
+    InnerState<T>* st = a.st;
+    if (!init && st->done) {
+        if (has_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
+        return;
+    }
+    const int k = init ? 0 : st->itn + 1;
+    const int c = st->p_c;
+    MlPostRow<T, NC> row{a, NC == 0 ? ((k & 1) ? a.z1 : a.z0) : a.wv, c, {}};
+    slices_only_gather<T>(a.rs, a.ml_x1, row, a.trim);
+    __shared__ T red[NA];
+    if (block_partials_arrive<T, NA>(row.acc, NA, a.partial, a.pstride, a.counter)) {
+        last_block_sum(a.partial, a.pstride, gridDim.x, NA, red, a.counter);
+        if (threadIdx.x == 0) {
+            double bb = (double)red[0];
+            for (int t = 0; t < c; ++t) {
+                const double h = (double)st->hv[t];
+                const double tv = a.dv[t] * h - (double)red[2 + t];
+                st->tv[t] = (T)tv;
+                bb += h * tv;
+            }
+            minres_step(a, st, (T)bb, NC == 0 ? red[1] : st->s_cur, init, k, cond, has_cond);
+        }
+    }
+}
+
 // z_{k+1} = w + Vh tv, its sum 1^T z_{k+1} (the next operator application's rank-one term) and
 // g_{k+1} = Vh^T z_{k+1} (its deflation term)
 template <typename T, int NC>
@@ -1190,13 +1322,22 @@ __global__ void __launch_bounds__(kThreads) k_ml_prep(InnerArgs<T> a, const doub
     }
 }
 
-// plain gather g = sum over the neighbours of x (the trimmed row gets 0); returns at once once the
-// inner solve has stopped (done != null)
+// gather g = sum over the neighbours of x (0 for the trimmed row), plus ob res where res is not null (the
+// V-cycle's residual, formed where the sum is); returns at once once the inner solve has stopped
+// (done != null)
+template <typename T>
+struct GatherResid {
+    const T* __restrict__ res;
+    T ob;
+    T* g;
+    __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) { g[r] = res ? ob * res[r] + s : s; }
+};
+
 template <typename T, int G, int TPB>
-__global__ void __launch_bounds__(TPB, TPB == kThreads ? 4 : 1) k_gather_vec(RowSched rs, const T* x, T* g,
-                                                                             int64_t skip, const int* done) {
+__global__ void __launch_bounds__(TPB, TPB == kThreads ? 4 : 1) k_gather_vec(RowSched rs, const T* x, const T* res, T ob,
+                                                                             T* g, int64_t skip, const int* done) {
     if (done && *done) return;
-    GatherStore<T> epi{g};
+    GatherResid<T> epi{res, ob, g};
     for_each_row_gather<T, G>(rs, x, epi, skip);
 }
 
@@ -1224,14 +1365,15 @@ __global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_phase1_gather_s
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_gather_vec_s(RowSched rs, const T* x, T* g,
-                                                                              int64_t skip, const int* done) {
+__global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_gather_vec_s(RowSched rs, const T* x, const T* res,
+                                                                              T ob, T* g, int64_t skip,
+                                                                              const int* done) {
     if (done && *done) return;
-    GatherStore<T> epi{g};
+    GatherResid<T> epi{res, ob, g};
     slices_only_gather<T>(rs, x, epi, skip);
 }
 
-inline int slice_grid(const RowSched& rs) {
+inline int slice_grid(const RowSched& rs, int ctas = kSliceBlocksPerSM) {
     static int nsm = 0;
     if (nsm == 0) {
         int dev = 0;
@@ -1239,7 +1381,7 @@ inline int slice_grid(const RowSched& rs) {
             nsm = 152;
     }
     const int64_t want = ((int64_t)rs.n_slices + kWarps - 1) / kWarps;
-    const int64_t cap = (int64_t)nsm * kSliceBlocksPerSM;
+    const int64_t cap = (int64_t)nsm * ctas;
     return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
@@ -1372,12 +1514,13 @@ void inner_phase2_cond(const InnerArgs<T>& a, cudaGraphConditionalHandle cond, c
 }
 
 template <typename T>
-void inner_gather_vec(const InnerArgs<T>& a, const T* x, T* g, int lanes, const int* done, cudaStream_t s) {
+void inner_gather_vec(const InnerArgs<T>& a, const T* x, const T* res, T ob, T* g, int lanes, const int* done,
+                      cudaStream_t s) {
     if (slices_only(a.rs)) {
-        k_gather_vec_s<T><<<slice_grid(a.rs), kThreads, 0, s>>>(a.rs, x, g, a.trim, done);
+        k_gather_vec_s<T><<<slice_grid(a.rs), kThreads, 0, s>>>(a.rs, x, res, ob, g, a.trim, done);
         return;
     }
-#define LGV(G, TPB) k_gather_vec<T, G, TPB><<<a.rs.grid(), TPB, a.rs.hub_bytes, s>>>(a.rs, x, g, a.trim, done)
+#define LGV(G, TPB) k_gather_vec<T, G, TPB><<<a.rs.grid(), TPB, a.rs.hub_bytes, s>>>(a.rs, x, res, ob, g, a.trim, done)
     ISIRA_GATHER_DISPATCH(lanes, a.rs.tpb, LGV);
 #undef LGV
 }
@@ -1385,6 +1528,51 @@ void inner_gather_vec(const InnerArgs<T>& a, const T* x, T* g, int lanes, const 
 template <typename T>
 void ml_inner_prep(const InnerArgs<T>& a, const double* R, const double* rnorm_dev, cudaStream_t s) {
     k_ml_prep<T><<<a.ew_blocks, kThreads, 0, s>>>(a, R, rnorm_dev);
+}
+
+// FP64 row kernels that reduce many values: a CTA's reduction costs as much FP64 issue time as hundreds of rows,
+// so each thread takes at least four row vectors before the grid grows beyond one CTA per SM
+// (613 x 487 grid, c = 3, phase 2c: 24.6 us at one vector per thread)
+template <typename T>
+inline int red_blocks(const InnerArgs<T>& a, const void* fn) {
+    const int g = wave_grid(fn, vec_blocks(a));
+    if (sizeof(T) == 4) return g;
+    const int nsm = std::max(1, wave_cache().nsm);
+    return std::min(g, std::max(nsm, (vec_blocks(a) + 3) / 4));
+}
+
+// gather and rows; graphs whose rows are all sliced take both in one kernel
+template <typename T>
+void ml_phase1_all(const InnerArgs<T>& a, int lanes, cudaStream_t s) {
+    if (slices_only(a.rs)) {
+        k_ml_phase1_s<T><<<slice_grid(a.rs, SlicedRows<T>::ctas), kThreads, 0, s>>>(a);
+        return;
+    }
+    inner_gather<T>(a, lanes, s);
+    ml_phase1<T>(a, s);
+}
+
+template <typename T>
+bool ml_post_fused(const InnerArgs<T>& a) { return a.ml_fuse_post && a.c <= 8 && slices_only(a.rs); }
+
+// the rest of the iteration after ml_vcycle: W x1, post-smoothing and phase 2b, phase 2c
+template <typename T>
+void ml_finish_cycle(const InnerArgs<T>& a, int init, int lanes, cudaGraphConditionalHandle cond, int has_cond,
+                     cudaStream_t s) {
+    if (ml_post_fused(a)) {
+        const int grid = slice_grid(a.rs, SlicedRows<T>::ctas);
+        if (a.c == 0) {
+            k_ml_post_s<T, 0><<<grid, kThreads, 0, s>>>(a, init, cond, has_cond);
+            return;
+        }
+        k_ml_post_s<T, 8><<<grid, kThreads, 0, s>>>(a, init, cond, has_cond);
+    } else {
+        if (a.ml_fuse_post)
+            inner_gather_vec<T>(a, a.ml_x1, nullptr, T(0), const_cast<T*>(a.ml_wx1), lanes,
+                                init ? nullptr : &a.st->done, s);
+        ml_phase2b<T>(a, init, cond, has_cond, s);
+    }
+    ml_phase2c<T>(a, init, s);
 }
 
 template <typename T>
@@ -1412,15 +1600,14 @@ void ml_project(const InnerArgs<T>& a, int init, cudaStream_t s) {
 template <typename T>
 void ml_phase2b(const InnerArgs<T>& a, int init, cudaGraphConditionalHandle cond, int has_cond, cudaStream_t s) {
 #define L2(NC)                                                                                              \
-    k_ml_phase2b<T, NC><<<wave_grid((const void*)k_ml_phase2b<T, NC>, vec_blocks(a)), kThreads, 0, s>>>(a, init, \
-                                                                                                  cond, has_cond)
+    k_ml_phase2b<T, NC><<<red_blocks(a, (const void*)k_ml_phase2b<T, NC>), kThreads, 0, s>>>(a, init, cond, has_cond)
     ISIRA_NC_DISPATCH(a.c, L2);
 #undef L2
 }
 
 template <typename T>
 void ml_phase2c(const InnerArgs<T>& a, int init, cudaStream_t s) {
-#define L2(NC) k_ml_phase2c<T, NC><<<wave_grid((const void*)k_ml_phase2c<T, NC>, vec_blocks(a)), kThreads, 0, s>>>(a, init)
+#define L2(NC) k_ml_phase2c<T, NC><<<red_blocks(a, (const void*)k_ml_phase2c<T, NC>), kThreads, 0, s>>>(a, init)
     ISIRA_NC_DISPATCH(a.c, L2);
 #undef L2
 }
@@ -1471,9 +1658,12 @@ void copy_vcol(const double* src, T* dst, int64_t n, cudaStream_t s) {
 #define ISIRA_INSTANTIATE_INNER(T)                                                                        \
     template void inner_phase1<T>(const InnerArgs<T>&, int, cudaStream_t);                               \
     template void inner_apply<T>(const InnerArgs<T>&, int, const int32_t*, T*, cudaStream_t);            \
-    template void inner_gather_vec<T>(const InnerArgs<T>&, const T*, T*, int, const int*, cudaStream_t);   \
+    template void inner_gather_vec<T>(const InnerArgs<T>&, const T*, const T*, T, T*, int, const int*, cudaStream_t); \
     template void ml_inner_prep<T>(const InnerArgs<T>&, const double*, const double*, cudaStream_t);      \
     template void ml_phase1<T>(const InnerArgs<T>&, cudaStream_t);                                       \
+    template void ml_phase1_all<T>(const InnerArgs<T>&, int, cudaStream_t);                              \
+    template bool ml_post_fused<T>(const InnerArgs<T>&);                                                 \
+    template void ml_finish_cycle<T>(const InnerArgs<T>&, int, int, cudaGraphConditionalHandle, int, cudaStream_t); \
     template void ml_phase2a<T>(const InnerArgs<T>&, int, cudaStream_t);                                 \
     template void ml_project<T>(const InnerArgs<T>&, int, cudaStream_t);                                 \
     template void ml_phase2b<T>(const InnerArgs<T>&, int, cudaGraphConditionalHandle, int, cudaStream_t); \

@@ -32,7 +32,7 @@ struct MlLevel {
     int64_t* mrp = nullptr;                   // members of each cluster of the next level
     int32_t* mem = nullptr;
     T* b = nullptr;                           // right-hand side of this level (levels >= 1)
-    T* x0 = nullptr; T* x1 = nullptr; T* x = nullptr;   // work vectors
+    T* x0 = nullptr; T* x1 = nullptr; T* x = nullptr;   // work vectors (levels >= 1: x0 holds D^{-1} b)
 };
 
 template <typename T>
@@ -43,9 +43,9 @@ struct MlHierarchy {
     T* inv = nullptr;                         // dense inverse of the coarsest level
 };
 
-// g = sum over the neighbours of x (level 0), on stream s
+// g = sum over the neighbours of x (level 0), plus (1 - omega) res where res is not null, on stream s
 template <typename T>
-using GatherFn = std::function<void(const T* x, T* g, cudaStream_t s)>;
+using GatherFn = std::function<void(const T* x, const T* res, T* g, cudaStream_t s)>;
 
 template <typename T>
 cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci, const double* d_w, int64_t n,
@@ -54,8 +54,11 @@ template <typename T> void ml_free(MlHierarchy<T>& H);
 // out = M^{-1} b, one V-cycle; kernels return at once while *done != 0 (done may be null)
 template <typename T>
 void ml_vcycle(MlHierarchy<T>& H, const T* b, T* out, const GatherFn<T>& gather, T omega, T alpha, const int* done,
-               bool x0_ready, bool skip_post0, cudaStream_t s);
+               bool x0_ready, bool skip_post0, const int32_t* perm, cudaStream_t s);
 template <typename T> int ml_launches(const MlHierarchy<T>& H, bool x0_ready, bool skip_post0);
+// b and level 0's x0 from the caller's x (perm: the caller's numbering; null: the solver's); nlev >= 2
+template <typename T>
+void ml_stage(MlHierarchy<T>& H, const T* x, const int32_t* perm, T omega, T* b, cudaStream_t s);
 
 // ------------------------------------------------------------------ inner solve
 // State of one preconditioned MINRES solve (Paige & Saunders 1975) kept in device
@@ -140,11 +143,16 @@ template <typename T> void gram_setup(const InnerArgs<T>& a, double* G_out, doub
                                       cudaStream_t s);
 template <typename T> void copy_vcol(const double* src, T* dst, int64_t n, cudaStream_t s);
 // multilevel-preconditioned MINRES (inner_impl.cuh)
-template <typename T> void inner_gather_vec(const InnerArgs<T>& a, const T* x, T* g, int lanes, const int* done,
-                                            cudaStream_t s);
+template <typename T> void inner_gather_vec(const InnerArgs<T>& a, const T* x, const T* res, T ob, T* g, int lanes,
+                                            const int* done, cudaStream_t s);
 template <typename T> void ml_inner_prep(const InnerArgs<T>& a, const double* R, const double* rnorm_dev,
                                          cudaStream_t s);
 template <typename T> void ml_phase1(const InnerArgs<T>& a, cudaStream_t s);
+template <typename T> void ml_phase1_all(const InnerArgs<T>& a, int lanes, cudaStream_t s);
+// whether the V-cycle's last gather, phase 2b and (c = 0) phase 2c run as one kernel
+template <typename T> bool ml_post_fused(const InnerArgs<T>& a);
+template <typename T> void ml_finish_cycle(const InnerArgs<T>& a, int init, int lanes, cudaGraphConditionalHandle cond,
+                                           int has_cond, cudaStream_t s);
 template <typename T> void ml_phase2a(const InnerArgs<T>& a, int init, cudaStream_t s);
 template <typename T> void ml_project(const InnerArgs<T>& a, int init, cudaStream_t s);
 template <typename T> void ml_phase2b(const InnerArgs<T>& a, int init, cudaGraphConditionalHandle cond, int has_cond,

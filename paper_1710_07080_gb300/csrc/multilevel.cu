@@ -21,12 +21,10 @@
 // matrix is diag(d) - W), 1/d, the cluster map of level l-1 (fine vertex -> cluster) and the member
 // lists of the clusters (CSR over the clusters).  Level 0 uses the solver's own gather for W x.
 //
-// Launches of one V-cycle: level 0 takes the gather twice (W x0 and W x1) with a restriction and a
-// prolongation / post-smoothing kernel around them (x0 itself usually comes from the caller's
-// projection kernel); each level l >= 1 takes one fused kernel down and one up, forming x0 and x1 of
-// the neighbours on the fly instead of storing them; the two coarsest levels, when small, run as
-// one CTA (k_ml_tail).  Five levels (the 128^3 grid: 2.1M, 264K, 15K, 690, 38 vertices) take 9
-// launches when the caller forms x0 and does level 0's post-smoothing in its own kernels.
+// Launches of one V-cycle: level 0 takes the gather twice (W x0 with the residual, W x1) with a restriction
+// and a prolongation / post-smoothing around them (x0, and the last gather with the post-smoothing, usually come
+// with the caller's own kernels); each level l >= 1 takes one kernel down and one up, and the
+// coarsest level one product with its dense inverse.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -218,116 +216,201 @@ __global__ void __launch_bounds__(kThreads) k_ml_scale(const T* __restrict__ b, 
         x[i] = i == skip ? T(0) : om * b[i] * dinv[i];
 }
 
-// bc[I] = sum over the members i of cluster I of (ob * b_i + add_i): level 0 passes ob = 1 - w and
-// add = W x0 (the gather), so the summand is the residual (1 - w) b + W x0; coarser levels pass ob = 0
-// and add = their residual.  One thread per cluster.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_ml_restrict(const T* __restrict__ b, const T* __restrict__ add, T ob,
-                                                          const int64_t* __restrict__ mrp,
+__global__ void __launch_bounds__(kThreads) k_ml_stage(const T* __restrict__ x, const int32_t* __restrict__ perm,
+                                                       const T* __restrict__ dinv, T om, int64_t n, int64_t skip,
+                                                       T* __restrict__ b, T* __restrict__ x0) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const T v = x[perm ? perm[i] : i];
+        b[i] = v;
+        x0[i] = i == skip ? T(0) : om * v * dinv[i];
+    }
+}
+
+// Level 0 -> 1: bc[I] = sum over the members i of cluster I of the residual res_i = (1 - w) b_i + (W x0)_i that the
+// gather stored, and qc = bc / dc for level 1's first smoothing step (null: level 1 is the coarsest).
+// One thread per cluster, four member indices and then four residuals in flight, added in member order:
+// the sums on the way down cancel (the trimmed Laplacian is nearly singular), so their order shows in FP32.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_ml_restrict(const T* __restrict__ res, const int64_t* __restrict__ mrp,
                                                           const int32_t* __restrict__ mem, int64_t nc,
-                                                          T* __restrict__ bc, const int* __restrict__ done) {
+                                                          T* __restrict__ bc, const T* __restrict__ dinvc,
+                                                          T* __restrict__ qc, const int* __restrict__ done) {
     if (done && *done) return;
     for (int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; I < nc; I += (int64_t)gridDim.x * blockDim.x) {
         T s = T(0);
-        for (int64_t q = mrp[I]; q < mrp[I + 1]; ++q) {
-            const int32_t i = mem[q];
-            s += ob * b[i] + add[i];
+        const int64_t end = mrp[I + 1];
+        for (int64_t q = mrp[I]; q < end; q += 4) {
+            int32_t i[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) i[u] = q + u < end ? mem[q + u] : -1;
+            T v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = i[u] >= 0 ? res[i[u]] : T(0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s += v[u];
         }
         bc[I] = s;
+        if (qc) qc[I] = s * dinvc[I];
     }
 }
 
-// x1 = x0 + a xc[agg(i)] (x0 = w D^{-1} b recomputed); the excluded vertex stays 0
+// level 0: x1 = x0 + a xc[agg(i)]; the excluded vertex stays 0
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_ml_prolong(const T* __restrict__ b, const T* __restrict__ dinv,
-                                                         const int32_t* __restrict__ agg, const T* __restrict__ xc,
-                                                         T om, T alpha, int64_t n, T* __restrict__ x1,
-                                                         const int* __restrict__ done) {
+__global__ void __launch_bounds__(kThreads) k_ml_prolong(const T* __restrict__ x0, const int32_t* __restrict__ agg,
+                                                         const T* __restrict__ xc, T alpha, int64_t n,
+                                                         T* __restrict__ x1, const int* __restrict__ done) {
     if (done && *done) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t I = agg[i];
-        x1[i] = I < 0 ? T(0) : om * b[i] * dinv[i] + alpha * xc[I];
+        x1[i] = I < 0 ? T(0) : x0[i] + alpha * xc[I];
     }
 }
 
-// post-smoothing: out = x1 + w D^{-1} (b - d x1 + W x1); level 0 takes (W x1) from the gather
+// level 0's post-smoothing: out = x1 + w D^{-1} (b - d x1 + W x1), (W x1) from the gather; out in the caller's
+// numbering if perm is given
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_ml_post(const T* __restrict__ b, const T* __restrict__ dinv,
                                                       const T* __restrict__ x1, const T* __restrict__ wx1, T om,
                                                       int64_t n, int64_t skip, T* __restrict__ out,
+                                                      const int32_t* __restrict__ perm,
                                                       const int* __restrict__ done) {
     if (done && *done) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (i == skip) {
-            out[i] = T(0);
-            continue;
-        }
         const T xi = x1[i], di = dinv[i];
-        out[i] = xi + om * (b[i] * di - xi + wx1[i] * di);
+        const T x = xi + om * (b[i] * di - xi + wx1[i] * di);
+        out[perm ? perm[i] : i] = i == skip ? T(0) : x;
     }
+}
+
+// Levels l >= 1 (no excluded vertex there).  The rows are ordered by cluster (ml_build), so the members of
+// cluster I are the rows mrp[I] .. mrp[I+1]-1 and their entries one contiguous CSR range.  Every level's
+// q = D^{-1} b (x0 = w q) is written by the kernel that forms its b, and its x1 = x0 + a P xc by the kernel that
+// forms xc (a coarse row writes its members), so a sweep gathers one vector and a level takes two launches:
+//   down  bc[I] = sum_{i in I} ((1 - w) b_i + w sum_{c in N(i)} w_ic q_c)     (restricted residual)
+//   up    out_i = x1_i + w (b_i - d_i x1_i + sum_c w_ic x1_c) / d_i
+// Both are bound by the latency of their index -> value chains, so a lane keeps four in flight.
+// (Forming x0 and x1 of the neighbours per entry instead cost two and three gathers: 12.1 and 14.3 us a
+// sweep on the 118 x 109 x 101 grid's level 1.)
+
+// stores x1 of the level below for the members of row I: x1_i = w q_i + alpha xI; G lanes (j of G)
+template <typename T>
+__device__ __forceinline__ void ml_store_members(const int64_t* __restrict__ mrp, const T* __restrict__ q, T om, T alpha,
+                                                 T xI, int64_t I, int j, int G, T* __restrict__ x1) {
+    for (int64_t i = mrp[I] + j; i < mrp[I + 1]; i += G) x1[i] = om * q[i] + alpha * xI;
 }
 
 // coarsest level: x = A^{-1} b with the dense inverse, one warp per row (the inverse is symmetric,
 // so row i is column i: coalesced)
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_ml_dense(const T* __restrict__ inv, const T* __restrict__ b, int64_t n,
-                                                       T* __restrict__ x, const int* __restrict__ done) {
+                                                       T* __restrict__ x, const int64_t* __restrict__ mrp,
+                                                       const T* __restrict__ q, T om, T alpha, T* __restrict__ x1,
+                                                       const int* __restrict__ done) {
     if (done && *done) return;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = w0; i < n; i += nw) {
         T s = T(0);
+#pragma unroll 4
         for (int64_t j = lane; j < n; j += 32) s += inv[j + i * n] * b[j];
         s = warp_sum(s);
         if (lane == 0) x[i] = s;
+        if (x1) ml_store_members(mrp, q, om, alpha, s, i, lane, 32, x1);
     }
 }
 
-// Fused kernels of the levels l >= 1 (no excluded vertex there).  With x0 = w D^{-1} b formed on the
-// fly for every neighbour, the down sweep of a level is one kernel and so is the up sweep:
-//   down  bc[I] = sum_{i in I} ((1 - w) b_i + w sum_{c in N(i)} w_ic b_c / d_c)      (restricted residual)
-//   up    x1_i = w b_i / d_i + a xc[agg_i],  out_i = x1_i + w (b_i - d_i x1_i + sum_c w_ic x1_c) / d_i
-// On levels l >= 1 the rows are ordered by cluster (ml_build), so the members of cluster I are the
-// rows mrp[I] .. mrp[I+1]-1 and their entries one contiguous CSR range: one warp per cluster, lanes
-// striding over the rows and over the entries (coalesced), G lanes per row in the up sweep.
-// x0 / x1 (FP64 only, else null): the level's x0 = w D^{-1} b / x1 stored by a separate kernel, read
-// instead of formed per entry: on this part an FP64 multiply costs as much as a load, so the FP64
-// path stores the vectors and the FP32 path forms them on the fly.
+// one warp per cluster, lanes striding over its rows and its entries (coalesced)
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_ml_down(const T* __restrict__ b, const T* __restrict__ dinv,
-                                                      const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                                      const T* __restrict__ w, const int64_t* __restrict__ mrp,
-                                                      T om, int64_t nc, T* __restrict__ bc,
-                                                      const T* __restrict__ x0, const int* __restrict__ done) {
+__global__ void __launch_bounds__(kThreads) k_ml_down(const T* __restrict__ b, const int32_t* __restrict__ rp,
+                                                      const int32_t* __restrict__ ci, const T* __restrict__ w,
+                                                      const int64_t* __restrict__ mrp, const T* __restrict__ qv, T om,
+                                                      int64_t nc, T* __restrict__ bc, const T* __restrict__ dinvc,
+                                                      T* __restrict__ qc, const int* __restrict__ done) {
     if (done && *done) return;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t I = w0; I < nc; I += nw) {
         const int64_t r_beg = mrp[I], r_end = mrp[I + 1];
+        const int32_t e_end = rp[r_end];
         T own = T(0), s = T(0);
         for (int64_t i = r_beg + lane; i < r_end; i += 32) own += b[i];
-        if (x0) {
-            for (int32_t e = rp[r_beg] + lane; e < rp[r_end]; e += 32) s += w[e] * x0[ci[e]];
-        } else {
-            for (int32_t e = rp[r_beg] + lane; e < rp[r_end]; e += 32) {
-                const int32_t c = ci[e];
-                s += w[e] * (b[c] * dinv[c]);
+        for (int32_t e = rp[r_beg] + lane; e < e_end; e += 128) {
+            int32_t c[4];
+            T v[4], q[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool ok = e + 32 * u < e_end;
+                c[u] = ok ? ci[e + 32 * u] : -1;
+                q[u] = ok ? w[e + 32 * u] : T(0);
             }
-            s *= om;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = c[u] >= 0 ? qv[c[u]] : T(0);
+            s += q[0] * v[0];
+            s += q[1] * v[1];
+            if (e - lane + 64 < e_end) {
+                s += q[2] * v[2];
+                s += q[3] * v[3];
+            }
         }
+        s *= om;
         const T acc = warp_sum((T(1) - om) * own + s);
+        if (lane == 0) {
+            bc[I] = acc;
+            if (qc) qc[I] = acc * dinvc[I];
+        }
+    }
+}
+
+// The same for a small level above the coarsest (at most kMlRowsMax rows): one warp per cluster, a lane per
+// member row, its entries in order.  Few clusters leave the entry-strided form short of warps, and the
+// row's own residual is what the sums on the way down are made of.
+constexpr int kMlRowsMax = 4096;
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_ml_down_rows(const T* __restrict__ b, const int32_t* __restrict__ rp,
+                                                           const int32_t* __restrict__ ci, const T* __restrict__ w,
+                                                           const int64_t* __restrict__ mrp, const T* __restrict__ qv,
+                                                           T om, int64_t nc, T* __restrict__ bc,
+                                                           const int* __restrict__ done) {
+    if (done && *done) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t I = w0; I < nc; I += nw) {
+        T acc = T(0);
+        for (int64_t i = mrp[I] + lane; i < mrp[I + 1]; i += 32) {
+            T s = T(0);
+            const int32_t e_end = rp[i + 1];
+            for (int32_t e = rp[i]; e < e_end; e += 4) {
+                int32_t c[4];
+                T v[4], q[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    c[u] = e + u < e_end ? ci[e + u] : -1;
+                    q[u] = e + u < e_end ? w[e + u] : T(0);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = c[u] >= 0 ? qv[c[u]] : T(0);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s += q[u] * v[u];
+            }
+            acc += (T(1) - om) * b[i] + om * s;
+        }
+        acc = warp_sum(acc);
         if (lane == 0) bc[I] = acc;
     }
 }
 
+// G lanes per row; out (level 1: the prolongation to level 0 reads it) or the members' x1 one level below
 template <typename T, int G>
 __global__ void __launch_bounds__(kThreads) k_ml_up(const T* __restrict__ b, const T* __restrict__ dinv,
-                                                    const int32_t* __restrict__ agg, const T* __restrict__ xc,
                                                     const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                                    const T* __restrict__ w, T om, T alpha, int64_t n,
-                                                    T* __restrict__ out, const T* __restrict__ x1v,
+                                                    const T* __restrict__ w, const T* __restrict__ x1, T om, T alpha,
+                                                    int64_t n, T* __restrict__ out, const int64_t* __restrict__ mrp,
+                                                    const T* __restrict__ qf, T* __restrict__ x1f,
                                                     const int* __restrict__ done) {
     if (done && *done) return;
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -337,78 +420,33 @@ __global__ void __launch_bounds__(kThreads) k_ml_up(const T* __restrict__ b, con
     for (int64_t p = 0; p < passes; ++p) {
         const int64_t row = g0 + p * groups;
         const bool valid = row < n;
-        T s = T(0);
+        T s0 = T(0), s1 = T(0);
         if (valid) {
-            if (x1v) {
-                for (int32_t e = rp[row] + j; e < rp[row + 1]; e += G) s += w[e] * x1v[ci[e]];
-            } else {
-                for (int32_t e = rp[row] + j; e < rp[row + 1]; e += G) {
-                    const int32_t c = ci[e];
-                    s += w[e] * (om * b[c] * dinv[c] + alpha * xc[agg[c]]);
+            const int32_t e_end = rp[row + 1];
+            for (int32_t e = rp[row] + j; e < e_end; e += 4 * G) {
+                int32_t c[4];
+                T v[4], q[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool ok = e + G * u < e_end;
+                    c[u] = ok ? ci[e + G * u] : -1;
+                    q[u] = ok ? w[e + G * u] : T(0);
                 }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = c[u] >= 0 ? x1[c[u]] : T(0);
+                s0 += q[0] * v[0] + q[1] * v[1];
+                s1 += q[2] * v[2] + q[3] * v[3];
             }
         }
+        T s = s0 + s1;
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-        if (valid && j == 0) {
-            const T bi = b[row], di = dinv[row];
-            const T x1 = x1v ? x1v[row] : om * bi * di + alpha * xc[agg[row]];
-            out[row] = x1 + om * (bi * di - x1 + s * di);
+        if (valid) {
+            const T di = dinv[row], xi = x1[row];
+            const T x = xi + om * (b[row] * di - xi + s * di);
+            if (x1f) ml_store_members(mrp, qf, om, alpha, x, row, j, G, x1f);
+            else if (j == 0) out[row] = x;
         }
-    }
-}
-
-// The two coarsest levels in one CTA: level t (n_t <= kMlTailMax rows, its CSR) and the dense
-// coarsest level t + 1.  Restricted residual of t, dense solve, prolongation and post-smoothing of t,
-// with the level-t vectors in shared memory; writes level t's output.
-constexpr int kMlTailMax = 4096;
-constexpr int kMlTailThreads = 1024;
-
-template <typename T>
-__global__ void __launch_bounds__(kMlTailThreads) k_ml_tail(const T* __restrict__ b, const T* __restrict__ dinv,
-                                                            const int32_t* __restrict__ rp,
-                                                            const int32_t* __restrict__ ci, const T* __restrict__ w,
-                                                            const int32_t* __restrict__ agg,
-                                                            const int64_t* __restrict__ mrp,
-                                                            const int32_t* __restrict__ mem,
-                                                            const T* __restrict__ inv, T om, T alpha, int nt, int nc,
-                                                            T* __restrict__ out, const int* __restrict__ done) {
-    if (done && *done) return;
-    extern __shared__ __align__(16) unsigned char tail_sm[];
-    T* r = reinterpret_cast<T*>(tail_sm);        // nt: residual, then x1
-    T* bc = r + nt;                              // nc
-    T* xc = bc + nc;                             // nc
-    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
-    for (int i = tid; i < nt; i += blockDim.x) {
-        T s = T(0);
-        for (int32_t e = rp[i]; e < rp[i + 1]; ++e) {
-            const int32_t c = ci[e];
-            s += w[e] * (b[c] * dinv[c]);
-        }
-        r[i] = (T(1) - om) * b[i] + om * s;
-    }
-    __syncthreads();
-    for (int I = wp; I < nc; I += blockDim.x / 32) {
-        T acc = T(0);
-        for (int64_t q = mrp[I] + lane; q < mrp[I + 1]; q += 32) acc += r[mem[q]];
-        acc = warp_sum(acc);
-        if (lane == 0) bc[I] = acc;
-    }
-    __syncthreads();
-    for (int I = wp; I < nc; I += blockDim.x / 32) {
-        T acc = T(0);
-        for (int J = lane; J < nc; J += 32) acc += inv[J + (int64_t)I * nc] * bc[J];
-        acc = warp_sum(acc);
-        if (lane == 0) xc[I] = acc;
-    }
-    __syncthreads();
-    for (int i = tid; i < nt; i += blockDim.x) r[i] = om * b[i] * dinv[i] + alpha * xc[agg[i]];
-    __syncthreads();
-    for (int i = tid; i < nt; i += blockDim.x) {
-        T s = T(0);
-        for (int32_t e = rp[i]; e < rp[i + 1]; ++e) s += w[e] * r[ci[e]];
-        const T x1 = r[i], di = dinv[i];
-        out[i] = x1 + om * (b[i] * di - x1 + s * di);
     }
 }
 
@@ -580,78 +618,71 @@ static int ml_group_grid(int64_t n, int G) {
 
 constexpr int kMlLanes = 4;          // lanes per coarse CSR row
 
-// Whether the two coarsest levels run as one k_ml_tail CTA.
-template <typename T>
-static bool ml_use_tail(const MlHierarchy<T>& H) {
-    return H.nlev >= 3 && H.lev[H.nlev - 2].n <= kMlTailMax && H.n_coarse <= kMlTailMax;
-}
-
 // out = M^{-1} b (b on level 0, n-space, the trimmed entry ignored; out may alias nothing else).
-// gather(x, g) must compute g = sum over neighbours of x for level 0 (the solver's gather).
+// gather(x, res, g) must compute g = W x (+ (1 - omega) res, if res is not null) for level 0.
 // x0_ready: level 0's x0 = w D^{-1} b is already in H.lev[0].x0 (written by the caller's kernel).
-// skip_post0 (nlev >= 2): stop after the gather of x1 (W x1 in H.lev[0].x0); the caller's next kernel
-// does level 0's post-smoothing (out is then not written).
+// skip_post0 (nlev >= 2): stop before the gather of x1 (H.lev[0].x1) that the caller's next kernels make, with
+// level 0's post-smoothing (out is then not written).
 template <typename T>
 void ml_vcycle(MlHierarchy<T>& H, const T* b, T* out, const GatherFn<T>& gather, T omega, T alpha, const int* done,
-               bool x0_ready, bool skip_post0, cudaStream_t s) {
+               bool x0_ready, bool skip_post0, const int32_t* perm, cudaStream_t s) {
     const int L = H.nlev;
+    MlLevel<T>& F = H.lev[0];
     if (L == 1) {
-        k_ml_dense<T><<<ml_warp_grid(H.lev[0].n), kThreads, 0, s>>>(H.inv, b, H.lev[0].n, out, done);
+        k_ml_dense<T><<<ml_warp_grid(F.n), kThreads, 0, s>>>(H.inv, b, F.n, out, nullptr, nullptr, omega, alpha,
+                                                             nullptr, done);
         return;
     }
-    const bool tail = ml_use_tail(H);
-    const int nmid = tail ? L - 3 : L - 2;        // levels 1..nmid take the fused down / up kernels
-    MlLevel<T>& F = H.lev[0];
-    // level 0 down: x0 = w D^{-1} b, its neighbour sums by the solver's gather, restricted residual
-    if (!x0_ready)
-        k_ml_scale<T><<<ml_grid(F.n), kThreads, 0, s>>>(b, F.dinv, omega, F.n, H.skip, F.x0, done);
-    gather(F.x0, F.x, s);                                            // F.x <- W x0
-    k_ml_restrict<T><<<ml_grid(H.lev[1].n), kThreads, 0, s>>>(b, F.x, T(1) - omega, F.mrp, F.mem, H.lev[1].n,
-                                                              H.lev[1].b, done);
-    constexpr bool store = sizeof(T) == 8;          // FP64: x0 and x1 stored, not formed per entry
-    for (int l = 1; l <= nmid; ++l) {
+    // level 0 down: x0 = w D^{-1} b, the residual (1 - w) b + W x0 in the solver's gather, restricted
+    if (!x0_ready) k_ml_scale<T><<<ml_grid(F.n), kThreads, 0, s>>>(b, F.dinv, omega, F.n, H.skip, F.x0, done);
+    gather(F.x0, b, F.x, s);
+    {
+        MlLevel<T>& C = H.lev[1];
+        k_ml_restrict<T><<<ml_grid(C.n), kThreads, 0, s>>>(F.x, F.mrp, F.mem, C.n, C.b, C.dinv,
+                                                          L > 2 ? C.x0 : nullptr, done);
+    }
+    for (int l = 1; l + 1 < L; ++l) {
         MlLevel<T>& D = H.lev[l];
         MlLevel<T>& C = H.lev[l + 1];
-        if (store) k_ml_scale<T><<<ml_grid(D.n), kThreads, 0, s>>>(D.b, D.dinv, omega, D.n, -1, D.x0, done);
-        k_ml_down<T><<<ml_warp_grid(C.n), kThreads, 0, s>>>(D.b, D.dinv, D.rp, D.ci, D.w, D.mrp, omega, C.n, C.b,
-                                                            store ? D.x0 : nullptr, done);
+        if (l + 2 == L && D.n <= kMlRowsMax)
+            k_ml_down_rows<T><<<ml_warp_grid(C.n), kThreads, 0, s>>>(D.b, D.rp, D.ci, D.w, D.mrp, D.x0, omega, C.n, C.b,
+                                                                     done);
+        else
+            k_ml_down<T><<<ml_warp_grid(C.n), kThreads, 0, s>>>(D.b, D.rp, D.ci, D.w, D.mrp, D.x0, omega, C.n, C.b,
+                                                                C.dinv, l + 2 < L ? C.x0 : nullptr, done);
     }
-    if (tail) {
-        static std::once_flag once;
-        std::call_once(once, [] {
-            cudaFuncSetAttribute(k_ml_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(T) * 3 * kMlTailMax));
-        });
-        MlLevel<T>& D = H.lev[L - 2];
-        const int nt = (int)D.n, nc = (int)H.n_coarse;
-        const int bytes = (int)(sizeof(T) * (nt + 2 * nc));
-        k_ml_tail<T><<<1, kMlTailThreads, bytes, s>>>(D.b, D.dinv, D.rp, D.ci, D.w, D.agg, D.mrp, D.mem, H.inv, omega,
-                                                      alpha, nt, nc, D.x, done);
-    } else {
+    {
         MlLevel<T>& C = H.lev[L - 1];
-        k_ml_dense<T><<<ml_warp_grid(C.n), kThreads, 0, s>>>(H.inv, C.b, C.n, C.x, done);
+        MlLevel<T>& D = H.lev[L - 2];
+        const bool below = L > 2;                                    // level L - 2 is not level 0
+        k_ml_dense<T><<<ml_warp_grid(C.n), kThreads, 0, s>>>(H.inv, C.b, C.n, C.x, D.mrp, D.x0, omega, alpha,
+                                                             below ? D.x1 : nullptr, done);
     }
-    for (int l = nmid; l >= 1; --l) {
+    for (int l = L - 2; l >= 1; --l) {
         MlLevel<T>& D = H.lev[l];
-        if (store)
-            k_ml_prolong<T><<<ml_grid(D.n), kThreads, 0, s>>>(D.b, D.dinv, D.agg, H.lev[l + 1].x, omega, alpha, D.n,
-                                                              D.x1, done);
-        k_ml_up<T, kMlLanes><<<ml_group_grid(D.n, kMlLanes), kThreads, 0, s>>>(D.b, D.dinv, D.agg, H.lev[l + 1].x, D.rp,
-                                                                                D.ci, D.w, omega, alpha, D.n, D.x,
-                                                                                store ? D.x1 : nullptr, done);
+        MlLevel<T>& B = H.lev[l - 1];
+        k_ml_up<T, kMlLanes><<<ml_group_grid(D.n, kMlLanes), kThreads, 0, s>>>(
+            D.b, D.dinv, D.rp, D.ci, D.w, D.x1, omega, alpha, D.n, D.x, B.mrp, B.x0, l > 1 ? B.x1 : nullptr, done);
     }
     // level 0 up: prolong, neighbour sums of x1, post-smooth
-    k_ml_prolong<T><<<ml_grid(F.n), kThreads, 0, s>>>(b, F.dinv, F.agg, H.lev[1].x, omega, alpha, F.n, F.x1, done);
-    gather(F.x1, F.x0, s);                                           // F.x0 <- W x1 (x0 is free now)
-    if (!skip_post0)
-        k_ml_post<T><<<ml_grid(F.n), kThreads, 0, s>>>(b, F.dinv, F.x1, F.x0, omega, F.n, H.skip, out, done);
+    k_ml_prolong<T><<<ml_grid(F.n), kThreads, 0, s>>>(F.x0, F.agg, H.lev[1].x, alpha, F.n, F.x1, done);
+    if (skip_post0) return;
+    gather(F.x1, nullptr, F.x0, s);                                  // F.x0 <- W x1 (x0 is free now)
+    k_ml_post<T><<<ml_grid(F.n), kThreads, 0, s>>>(b, F.dinv, F.x1, F.x0, omega, F.n, H.skip, out, perm, done);
 }
 
+// launches of one call (without the caller's gather of x1 when skip_post0)
 template <typename T>
 int ml_launches(const MlHierarchy<T>& H, bool x0_ready, bool skip_post0) {
     if (H.nlev <= 1) return 1;
-    const int nmid = ml_use_tail(H) ? H.nlev - 3 : H.nlev - 2;
-    return (x0_ready ? 0 : 1) + 2 + (sizeof(T) == 8 ? 4 : 2) * nmid + 1 + (skip_post0 ? 2 : 3);
+    return (x0_ready ? 0 : 1) + 2 + 2 * (H.nlev - 2) + 1 + 1 + (skip_post0 ? 0 : 2);
+}
+
+// b = x (the caller's vector and numbering) and level 0's x0 = w D^{-1} b
+template <typename T>
+void ml_stage(MlHierarchy<T>& H, const T* x, const int32_t* perm, T omega, T* b, cudaStream_t s) {
+    MlLevel<T>& F = H.lev[0];
+    k_ml_stage<T><<<ml_grid(F.n), kThreads, 0, s>>>(x, perm, F.dinv, omega, F.n, H.skip, b, F.x0);
 }
 
 #define ISIRA_INSTANTIATE_ML(T)                                                                              \
@@ -659,7 +690,8 @@ int ml_launches(const MlHierarchy<T>& H, bool x0_ready, bool skip_post0) {
                                      int64_t, int64_t, cudaStream_t);                                        \
     template void ml_free<T>(MlHierarchy<T>&);                                                               \
     template void ml_vcycle<T>(MlHierarchy<T>&, const T*, T*, const GatherFn<T>&, T, T, const int*, bool,     \
-                               bool, cudaStream_t);                                                          \
+                               bool, const int32_t*, cudaStream_t);                                          \
+    template void ml_stage<T>(MlHierarchy<T>&, const T*, const int32_t*, T, T*, cudaStream_t);               \
     template int ml_launches<T>(const MlHierarchy<T>&, bool, bool);
 ISIRA_INSTANTIATE_ML(float)
 ISIRA_INSTANTIATE_ML(double)

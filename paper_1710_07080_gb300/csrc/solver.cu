@@ -447,20 +447,32 @@ void ensure_ml(isira_handle h, InnerBuffers<T>& b) {
 template <typename T>
 T ml_alpha(isira_handle h) { return (T)(h->opts.ml_alpha > 0.0 ? h->opts.ml_alpha : 1.5); }
 
+// the V-cycle's gathers on the solver's graph: W x, or the residual (1 - omega) res + W x
+template <typename T>
+GatherFn<T> ml_gather(isira_handle h, const InnerArgs<T>& a, const int* done) {
+    return [h, &a, done](const T* x, const T* res, T* g, cudaStream_t st) {
+        inner_gather_vec<T>(a, x, res, T(1) - (T)kMlOmega, g, h->lanes, done, st);
+    };
+}
+
+// the iteration after phase 1 (init: the first preconditioned vector)
+template <typename T>
+void ml_second_phase(isira_handle h, InnerBuffers<T>& b, const InnerArgs<T>& a, int init,
+                     cudaGraphConditionalHandle cond, int has_cond, cudaStream_t s) {
+    const int* done = init ? nullptr : &a.st->done;
+    ml_phase2a<T>(a, init, s);
+    ml_project<T>(a, init, s);
+    ml_vcycle<T>(b.H, a.c > 0 ? a.rin : a.rcur, a.wv, ml_gather<T>(h, a, done), (T)kMlOmega, ml_alpha<T>(h), done,
+                 a.ml_x0 != nullptr, a.ml_fuse_post != 0, nullptr, s);
+    ml_finish_cycle<T>(a, init, h->lanes, cond, has_cond, s);
+}
+
 // body of one multilevel MINRES iteration (graph capture or chunked launches)
 template <typename T>
 void ml_iteration(isira_handle h, InnerBuffers<T>& b, const InnerArgs<T>& a, cudaGraphConditionalHandle cond,
                   int has_cond, cudaStream_t s) {
-    const int* done = &a.st->done;
-    GatherFn<T> gather = [&](const T* x, T* g, cudaStream_t st) { inner_gather_vec<T>(a, x, g, h->lanes, done, st); };
-    inner_gather<T>(a, h->lanes, s);
-    ml_phase1<T>(a, s);
-    ml_phase2a<T>(a, 0, s);
-    ml_project<T>(a, 0, s);
-    ml_vcycle<T>(b.H, a.c > 0 ? a.rin : a.rcur, a.wv, gather, (T)kMlOmega, ml_alpha<T>(h), done,
-                 a.c > 0 && a.ml_x0 != nullptr, a.ml_fuse_post != 0, s);
-    ml_phase2b<T>(a, 0, cond, has_cond, s);
-    ml_phase2c<T>(a, 0, s);
+    ml_phase1_all<T>(a, h->lanes, s);
+    ml_second_phase<T>(h, b, a, 0, cond, has_cond, s);
 }
 
 template <typename T>
@@ -488,8 +500,10 @@ cudaGraphExec_t build_ml_graph(isira_handle h, InnerBuffers<T>& b, const InnerAr
 }
 
 template <typename T>
-int ml_launches_per_iteration(const InnerBuffers<T>& b, int c) {
-    return 6 + (c > 0 ? 1 : 0) + ml_launches(b.H, c > 0 && b.H.nlev >= 2, b.H.nlev >= 2);
+int ml_launches_per_iteration(const InnerBuffers<T>& b, const InnerArgs<T>& a) {
+    const bool multi = b.H.nlev >= 2, fused = ml_post_fused(a);
+    return (slices_only(a.rs) ? 1 : 2) + 1 + (a.c > 0 ? 1 : 0) + ml_launches(b.H, multi, multi) +
+           (fused ? 1 : multi ? 2 : 1) + (fused && a.c == 0 ? 0 : 1);
 }
 
 // One inner solve with the multilevel preconditioner; same contract as run_inner.  lam: the
@@ -501,7 +515,6 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
     ensure_ml(h, b);
     InnerArgs<T> a = make_args<T>(h, b, sigma, c, Vt, ldv, tau, max_it);
     cudaStream_t s = h->stream;
-    GatherFn<T> gather0 = [&](const T* x, T* g, cudaStream_t st) { inner_gather_vec<T>(a, x, g, h->lanes, nullptr, st); };
     if (c > 0 && gram_dirty) {
         // D = diag(1 / (lambda_t - sigma + delta)) for the deflated directions (pageable copy: synchronous)
         double dv[kCMax];
@@ -511,13 +524,8 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
     const bool ahead = !allow_graph && h->opts.inner_graph && !h->profiling && !h->sync_ev;
     if (ahead) reset_inner_status(h);
     ml_inner_prep<T>(a, R, rnorm_dev, s);
-    ml_phase2a<T>(a, 1, s);
-    ml_project<T>(a, 1, s);
-    ml_vcycle<T>(b.H, c > 0 ? a.rin : a.rcur, a.wv, gather0, (T)kMlOmega, ml_alpha<T>(h), nullptr,
-                 c > 0 && a.ml_x0 != nullptr, a.ml_fuse_post != 0, s);
-    ml_phase2b<T>(a, 1, cudaGraphConditionalHandle{}, 0, s);
-    ml_phase2c<T>(a, 1, s);
-    const int per_it = ml_launches_per_iteration(b, c);
+    ml_second_phase<T>(h, b, a, 1, cudaGraphConditionalHandle{}, 0, s);
+    const int per_it = ml_launches_per_iteration(b, a);
     h->stats.kernel_launches += per_it - 1;
     if (ahead) {
         const int nl = run_ahead(h, max_it, 2, [&] { ml_iteration<T>(h, b, a, cudaGraphConditionalHandle{}, 0, s); });
@@ -544,16 +552,12 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
         const bool prof = h->profiling != 0;
         for (int i = 0; i < chunk; ++i) {
             if (prof) ck(cudaEventRecord(h->ev[4 * i], s));
-            inner_gather<T>(a, h->lanes, s);
+            const bool one = slices_only(a.rs);          // gather and rows in one kernel
+            if (one) ml_phase1_all<T>(a, h->lanes, s); else inner_gather<T>(a, h->lanes, s);
             if (prof) ck(cudaEventRecord(h->ev[4 * i + 1], s));
-            ml_phase1<T>(a, s);
+            if (!one) ml_phase1<T>(a, s);
             if (prof) ck(cudaEventRecord(h->ev[4 * i + 2], s));
-            ml_phase2a<T>(a, 0, s);
-            ml_project<T>(a, 0, s);
-            ml_vcycle<T>(b.H, c > 0 ? a.rin : a.rcur, a.wv, gather0, (T)kMlOmega, ml_alpha<T>(h), &a.st->done,
-                         c > 0 && a.ml_x0 != nullptr, a.ml_fuse_post != 0, s);
-            ml_phase2b<T>(a, 0, cudaGraphConditionalHandle{}, 0, s);
-            ml_phase2c<T>(a, 0, s);
+            ml_second_phase<T>(h, b, a, 0, cudaGraphConditionalHandle{}, 0, s);
             if (prof) ck(cudaEventRecord(h->ev[4 * i + 3], s));
         }
         h->stats.spmv_launches += chunk;
@@ -887,14 +891,19 @@ void precond_apply_t(isira_handle h, InnerBuffers<T>& b, const T* d_x, T* d_y) {
     alloc_inner(h, b);
     ensure_ml(h, b);
     InnerArgs<T> a = make_args<T>(h, b, 0.0, 0, nullptr, h->ld, 1e-3, 1);
-    T* xin = a.rcur;
-    T* yout = a.wv;
-    if (h->perm) to_internal<T>(d_x, h->perm, h->n, xin, s);
-    else ck(cudaMemcpyAsync(xin, d_x, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
-    GatherFn<T> gather = [&](const T* x, T* g, cudaStream_t st) { inner_gather_vec<T>(a, x, g, h->lanes, nullptr, st); };
-    ml_vcycle<T>(b.H, xin, yout, gather, (T)kMlOmega, ml_alpha<T>(h), nullptr, false, false, s);
-    if (h->perm) to_external<T>(yout, h->perm, h->n, d_y, s);
-    else ck(cudaMemcpyAsync(d_y, yout, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
+    if (b.H.nlev >= 2) {
+        // the caller's numbering is left and met again inside the cycle's own first and last kernels
+        ml_stage<T>(b.H, d_x, h->perm, (T)kMlOmega, a.rcur, s);
+        ml_vcycle<T>(b.H, a.rcur, d_y, ml_gather<T>(h, a, nullptr), (T)kMlOmega, ml_alpha<T>(h), nullptr, true, false,
+                     h->perm, s);
+    } else {
+        if (h->perm) to_internal<T>(d_x, h->perm, h->n, a.rcur, s);
+        else ck(cudaMemcpyAsync(a.rcur, d_x, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
+        ml_vcycle<T>(b.H, a.rcur, a.wv, ml_gather<T>(h, a, nullptr), (T)kMlOmega, ml_alpha<T>(h), nullptr, false, false,
+                     nullptr, s);
+        if (h->perm) to_external<T>(a.wv, h->perm, h->n, d_y, s);
+        else ck(cudaMemcpyAsync(d_y, a.wv, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
+    }
     sync(h);
 }
 }  // namespace
