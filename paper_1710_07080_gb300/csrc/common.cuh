@@ -658,6 +658,25 @@ __device__ __forceinline__ void for_each_row_gather(const RowSched& S, const T* 
 // loaded ahead and eight independent index loads per pass.  Few registers, so a full SM of warps
 // keeps loads in flight.  A row's entries are added in slice order in two interleaved partial
 // sums, whatever the launch shape (the result does not depend on the grid).
+// The epilogue has two halves: pre(row) loads what it needs of the row's vectors before the gather, so
+// that those loads and the dependent index -> value chains are in flight together, and fin(row, loaded,
+// sum) does the arithmetic.  (Rows up to the next multiple of 32 are loaded: every vector has them.)
+// In FP64 the additions and multiplications stop at the slice's width: an SM issues an FP64 warp
+// instruction every 16 cycles, and a grid's four entries in eight slots cost twice what they need.
+template <typename T>
+__device__ __forceinline__ T pass_sum(const T (&v)[8], int r) {
+    T s = v[0];
+    if (r > 1) s += v[1];
+    if (r > 2) { T t = v[2]; if (r > 3) t += v[3]; s += t; }
+    if (r > 4) {
+        T t = v[4];
+        if (r > 5) t += v[5];
+        if (r > 6) { T q = v[6]; if (r > 7) q += v[7]; t += q; }
+        s += t;
+    }
+    return s;
+}
+
 template <typename T, class Epi>
 __device__ __forceinline__ void slices_only_gather(const RowSched& S, const T* __restrict__ x, Epi& epi, int64_t skip) {
     const int lane = threadIdx.x & 31;
@@ -670,6 +689,8 @@ __device__ __forceinline__ void slices_only_gather(const RowSched& S, const T* _
         const int64_t oa = o0;
         const int wa = (int)((o1 - o0) >> 5);
         if (s + nw < S.n_slices) { o0 = S.sell_off[s + nw]; o1 = S.sell_off[s + nw + 1]; }   // next slice
+        const int64_t row = S.light0 + (int64_t)s * 32 + lane;
+        const typename Epi::Pre pre = epi.pre(row);
         T s0 = 0, s1 = 0;
         for (int q = 0; q < wa; q += 8) {
             int32_t ia[8];
@@ -680,26 +701,36 @@ __device__ __forceinline__ void slices_only_gather(const RowSched& S, const T* _
             for (int u = 0; u < 8; ++u) va[u] = ia[u] >= 0 ? __ldg(x + ia[u]) : T(0);
             if (sw) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u) va[u] *= ia[u] >= 0 ? __ldcs(sw + oa + (int64_t)(q + u) * 32 + lane) : T(0);
+                for (int u = 0; u < 8; ++u)
+                    if (sizeof(T) == 4 || q + u < wa)
+                        va[u] *= ia[u] >= 0 ? __ldcs(sw + oa + (int64_t)(q + u) * 32 + lane) : T(0);
             }
-            s0 += (va[0] + va[1]) + (va[2] + va[3]);
-            s1 += (va[4] + va[5]) + (va[6] + va[7]);
+            if constexpr (sizeof(T) == 4) {
+                s0 += (va[0] + va[1]) + (va[2] + va[3]);
+                s1 += (va[4] + va[5]) + (va[6] + va[7]);
+            } else {
+                const T t = pass_sum(va, wa - q);
+                s0 = q == 0 ? t : s0 + t;
+            }
         }
-        const int64_t row = S.light0 + (int64_t)s * 32 + lane;
-        if (row < S.n) epi(row, 0, row == skip ? T(0) : s0 + s1);
+        if constexpr (sizeof(T) == 4) s0 += s1;
+        if (row < S.n) epi.fin(row, pre, row == skip ? T(0) : s0);
     }
-    if (skip >= 0 && skip < S.light0 && blockIdx.x == 0 && threadIdx.x == 0) epi(skip, 0, T(0));
 }
 
 // The slices-only kernels are used when every row is sliced: relabelling on, sliced copy on, no
-// work items.
+// work items (light0 = 0, so the skipped row, too, is in a slice).
 __host__ __device__ inline bool slices_only(const RowSched& S) { return S.sell && S.n_items == 0; }
-constexpr int kSliceBlocksPerSM = 8;
+// resident CTAs per SM of the plain sliced gathers (FP64 wants 40 registers)
+template <typename T> struct SliceBlocks { static constexpr int value = sizeof(T) == 4 ? 8 : 6; };
 
 // Epilogue of the plain gather: g[row] = sum over the row (0 for the skipped row).
 template <typename T>
 struct GatherStore {
     T* g;
+    struct Pre {};
+    __device__ __forceinline__ Pre pre(int64_t) const { return {}; }
+    __device__ __forceinline__ void fin(int64_t r, const Pre&, T s) { g[r] = s; }
     __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) { g[r] = s; }
 };
 

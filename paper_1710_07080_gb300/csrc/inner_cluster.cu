@@ -103,16 +103,7 @@ __device__ __forceinline__ T cl_total(const T* v) {
 template <typename T>
 __device__ __forceinline__ T cl_pass_sum(const T (&v)[8], int r) {
     if constexpr (sizeof(T) == 4) return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
-    T s = v[0];
-    if (r > 1) s += v[1];
-    if (r > 2) { T t = v[2]; if (r > 3) t += v[3]; s += t; }
-    if (r > 4) {
-        T t = v[4];
-        if (r > 5) t += v[5];
-        if (r > 6) { T q = v[6]; if (r > 7) q += v[7]; t += q; }
-        s += t;
-    }
-    return s;
+    return pass_sum(v, r);
 }
 
 }  // namespace

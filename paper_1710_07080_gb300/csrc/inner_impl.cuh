@@ -501,14 +501,17 @@ struct ApplyStore {
     int c;
     const int32_t* __restrict__ perm;
     T* yext;
-    __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) {
+    struct Pre { T z, deg; };
+    __device__ __forceinline__ Pre pre(int64_t r) const {
+        const T* dw = a.rs.template degw<T>();
+        return {a.z0[r], dw ? dw[r] : (T)a.deg[r]};
+    }
+    __device__ __forceinline__ void fin(int64_t r, const Pre& p, T s) {
         T v = T(0);
         if (r != a.trim) {
-            const T* dw = a.rs.template degw<T>();
-            const T degT = dw ? dw[r] : (T)a.deg[r];
             T vd = T(0);
             for (int t = 0; t < c; ++t) vd += a.Vt[(int64_t)t * a.ldv + r] * u1s[t];
-            v = ((degT - sigma) * a.z0[r] - s + s_term) + vd;
+            v = ((p.deg - sigma) * p.z - s + s_term) + vd;
         }
         yext[perm ? perm[r] : r] = v;
     }
@@ -846,7 +849,7 @@ __device__ __forceinline__ void ml_phase1_finish(const InnerArgs<T>& a, T acc0, 
 
 // resident CTAs per SM of the kernels that do row arithmetic in a sliced gather: FP32 wants the warps in
 // flight; in FP64 every CTA's reduction costs FP64 issue slots (a warp sum as much as five rows)
-template <typename T> struct SlicedRows { static constexpr int ctas = sizeof(T) == 4 ? 6 : 4; };
+template <typename T> struct SlicedRows { static constexpr int ctas = sizeof(T) == 4 ? 5 : 3; };
 
 template <typename T, int NC>
 __global__ void __launch_bounds__(kThreads) k_ml_phase1(InnerArgs<T> a) {
@@ -915,8 +918,7 @@ __global__ void __launch_bounds__(kThreads) k_ml_phase1(InnerArgs<T> a) {
 }
 
 // The same with the gather, for graphs whose rows are all sliced: a lane has its row's neighbour sum and
-// does the row at once, so the sums are neither stored nor read and a launch falls away (118 x 109 x 101
-// grid, FP32: 12 + 15.4 us as two kernels).
+// does the row at once, so the sums are neither stored nor read and a launch falls away.
 template <typename T>
 struct MlPhase1Row {
     const InnerArgs<T>& a;
@@ -928,20 +930,33 @@ struct MlPhase1Row {
     const T* __restrict__ dw;
     T sigma, s_term, inv_beta, inv_oldb, cprev, oldeps, dlt, inv_gamma, phi, acc;
     bool has_prev;
-    __device__ __forceinline__ void operator()(int64_t r, int64_t, T g) {
-        const bool ok = r != a.trim;
-        const T z = zc[r];
-        const T deg = dw ? dw[r] : (T)a.deg[r];
-        T y = ((deg - sigma) * z - g + s_term) * inv_beta;
+    struct Pre { T z, deg, rp, zp, w2, w1, x; };
+    __device__ __forceinline__ Pre pre(int64_t r) const {
+        Pre p;
+        p.z = zc[r];
+        p.deg = dw ? dw[r] : (T)a.deg[r];
+        p.rp = p.zp = p.w2 = p.w1 = p.x = T(0);
         if (has_prev) {
-            y -= cprev * a.rprev[r];
-            const T w = (zp[r] * inv_oldb - oldeps * wo2[r] - dlt * wo1[r]) * inv_gamma;
+            p.rp = a.rprev[r];
+            p.zp = zp[r];
+            p.w2 = wo2[r];
+            p.w1 = wo1[r];
+            p.x = a.x[r];
+        }
+        return p;
+    }
+    __device__ __forceinline__ void fin(int64_t r, const Pre& p, T g) {
+        const bool ok = r != a.trim;
+        T y = ((p.deg - sigma) * p.z - g + s_term) * inv_beta;
+        if (has_prev) {
+            y -= cprev * p.rp;
+            const T w = (p.zp * inv_oldb - oldeps * p.w2 - dlt * p.w1) * inv_gamma;
             wn[r] = ok ? w : T(0);
-            if (ok) a.x[r] += phi * w;
+            if (ok) a.x[r] = p.x + phi * w;
         }
         y = ok ? y : T(0);
         a.Y[r] = y;
-        acc += z * inv_beta * y;
+        acc += p.z * inv_beta * y;
     }
 };
 
@@ -1191,13 +1206,17 @@ struct MlPostRow {
     T* __restrict__ out;
     int c;
     T acc[2 + NE];                                     // r^T w, (c = 0) 1^T w, Vh^T w
-    __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) {
+    struct Pre { T x1, di, b, r; };
+    __device__ __forceinline__ Pre pre(int64_t r) const {
+        const T b = a.ml_b0[r];
+        return {a.ml_x1[r], a.ml_dinv0[r], b, NC == 0 ? b : a.rcur[r]};
+    }
+    __device__ __forceinline__ void fin(int64_t r, const Pre& p, T s) {
         const bool ok = r != a.trim;
-        const T x1 = a.ml_x1[r], di = a.ml_dinv0[r], b = a.ml_b0[r];
-        T w = x1 + a.ml_omega * (b * di - x1 + s * di);
+        T w = p.x1 + a.ml_omega * (p.b * p.di - p.x1 + s * p.di);
         w = ok ? w : T(0);
         out[r] = w;
-        acc[0] += (ok ? (NC == 0 ? b : a.rcur[r]) : T(0)) * w;
+        acc[0] += (ok ? p.r : T(0)) * w;
         if (NC == 0) acc[1] += w;
 #pragma unroll
         for (int t = 0; t < NE; ++t)
@@ -1330,7 +1349,10 @@ struct GatherResid {
     const T* __restrict__ res;
     T ob;
     T* g;
-    __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) { g[r] = res ? ob * res[r] + s : s; }
+    struct Pre { T v; };
+    __device__ __forceinline__ Pre pre(int64_t r) const { return {res ? res[r] : T(0)}; }
+    __device__ __forceinline__ void fin(int64_t r, const Pre& p, T s) { g[r] = res ? ob * p.v + s : s; }
+    __device__ __forceinline__ void operator()(int64_t r, int64_t, T s) { fin(r, pre(r), s); }
 };
 
 template <typename T, int G, int TPB>
@@ -1356,7 +1378,7 @@ __global__ void __launch_bounds__(TPB, TPB == kThreads ? 4 : 1) k_gather_vec(Row
 
 // slices-only gathers (every row in the sliced copy): z_k of the current iteration, or a given vector
 template <typename T>
-__global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_phase1_gather_s(InnerArgs<T> a) {
+__global__ void __launch_bounds__(kThreads, SliceBlocks<T>::value) k_phase1_gather_s(InnerArgs<T> a) {
     const InnerState<T>* st = a.st;
     if (st->done) return;
     const T* zc = (st->itn & 1) ? a.z1 : a.z0;
@@ -1365,7 +1387,7 @@ __global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_phase1_gather_s
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_gather_vec_s(RowSched rs, const T* x, const T* res,
+__global__ void __launch_bounds__(kThreads, SliceBlocks<T>::value) k_gather_vec_s(RowSched rs, const T* x, const T* res,
                                                                               T ob, T* g, int64_t skip,
                                                                               const int* done) {
     if (done && *done) return;
@@ -1373,7 +1395,7 @@ __global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_gather_vec_s(Ro
     slices_only_gather<T>(rs, x, epi, skip);
 }
 
-inline int slice_grid(const RowSched& rs, int ctas = kSliceBlocksPerSM) {
+inline int slice_grid(const RowSched& rs, int ctas) {
     static int nsm = 0;
     if (nsm == 0) {
         int dev = 0;
@@ -1388,7 +1410,7 @@ inline int slice_grid(const RowSched& rs, int ctas = kSliceBlocksPerSM) {
 template <typename T>
 void inner_gather(const InnerArgs<T>& a, int lanes, cudaStream_t s) {
     if (slices_only(a.rs)) {
-        k_phase1_gather_s<T><<<slice_grid(a.rs), kThreads, 0, s>>>(a);
+        k_phase1_gather_s<T><<<slice_grid(a.rs, SliceBlocks<T>::value), kThreads, 0, s>>>(a);
         return;
     }
 #define LG(G, TPB) k_phase1_gather<T, G, TPB><<<a.rs.grid(), TPB, a.rs.hub_bytes, s>>>(a)
@@ -1490,7 +1512,7 @@ void inner_phase1(const InnerArgs<T>& a, int lanes, cudaStream_t s) {
 template <typename T>
 void inner_apply(const InnerArgs<T>& a, int lanes, const int32_t* perm, T* y, cudaStream_t s) {
     if (slices_only(a.rs)) {
-        k_apply_slices<T><<<slice_grid(a.rs), kThreads, 0, s>>>(a, perm, y);
+        k_apply_slices<T><<<slice_grid(a.rs, 4), kThreads, 0, s>>>(a, perm, y);
         return;
     }
     inner_gather<T>(a, lanes, s);
@@ -1517,7 +1539,7 @@ template <typename T>
 void inner_gather_vec(const InnerArgs<T>& a, const T* x, const T* res, T ob, T* g, int lanes, const int* done,
                       cudaStream_t s) {
     if (slices_only(a.rs)) {
-        k_gather_vec_s<T><<<slice_grid(a.rs), kThreads, 0, s>>>(a.rs, x, res, ob, g, a.trim, done);
+        k_gather_vec_s<T><<<slice_grid(a.rs, SliceBlocks<T>::value), kThreads, 0, s>>>(a.rs, x, res, ob, g, a.trim, done);
         return;
     }
 #define LGV(G, TPB) k_gather_vec<T, G, TPB><<<a.rs.grid(), TPB, a.rs.hub_bytes, s>>>(a.rs, x, res, ob, g, a.trim, done)

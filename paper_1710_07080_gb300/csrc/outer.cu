@@ -973,7 +973,7 @@ __global__ void __launch_bounds__(kThreads) k_laplacian_rows(OuterArgs a, const 
         y[r] = row_degree<double>(a.rs, r) * x[r] - a.gsum[r];
 }
 
-__global__ void __launch_bounds__(kThreads, kSliceBlocksPerSM) k_gather_plain_s(RowSched rs, const double* x, double* g) {
+__global__ void __launch_bounds__(kThreads, SliceBlocks<double>::value) k_gather_plain_s(RowSched rs, const double* x, double* g) {
     GatherStore<double> epi{g};
     slices_only_gather<double>(rs, x, epi, -1);
 }
@@ -988,7 +988,7 @@ static void outer_gather(const OuterArgs& a, const double* x, int lanes, cudaStr
                 nsm = 152;
         }
         const int64_t want = ((int64_t)a.rs.n_slices + kWarps - 1) / kWarps;
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)nsm * kSliceBlocksPerSM));
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)nsm * SliceBlocks<double>::value));
         k_gather_plain_s<<<grid, kThreads, 0, s>>>(a.rs, x, a.gsum);
         return;
     }
