@@ -655,26 +655,48 @@ __device__ __forceinline__ void for_each_row_gather(const RowSched& S, const T* 
 
 // Gather for graphs without long rows (every row in the sliced copy, no work items): warp w walks
 // the slices w, w + W, ... (W warps in the grid), one lane per row, with the next slice's offsets
-// loaded ahead and eight independent index loads per pass.  Few registers, so a full SM of warps
-// keeps loads in flight.  A row's entries are added in slice order in two interleaved partial
+// loaded ahead and eight independent index loads per pass.  A slice's first indices are loaded while the
+// slice before it gathers, so a warp waits for one of the two latencies of the chain index -> value, not
+// for their sum.  A row's entries are added in slice order in two interleaved partial
 // sums, whatever the launch shape (the result does not depend on the grid).
 // The epilogue has two halves: pre(row) loads what it needs of the row's vectors before the gather, so
 // that those loads and the dependent index -> value chains are in flight together, and fin(row, loaded,
 // sum) does the arithmetic.  (Rows up to the next multiple of 32 are loaded: every vector has them.)
-// In FP64 the additions and multiplications stop at the slice's width: an SM issues an FP64 warp
-// instruction every 16 cycles, and a grid's four entries in eight slots cost twice what they need.
+// In FP64 the arithmetic stops at the slice's width: an SM issues an FP64 warp instruction every 16 cycles,
+// and a grid's four entries in eight slots cost twice what they need.  The widths are cases of a switch,
+// since the compiler turns short conditional blocks into predicated instructions, and a predicated-off
+// FP64 instruction takes its 16 cycles all the same (2000 passes of width 3: 955 us as a switch, 1249 us as
+// nested conditions, 2489 us at full width).
 template <typename T>
 __device__ __forceinline__ T pass_sum(const T (&v)[8], int r) {
-    T s = v[0];
-    if (r > 1) s += v[1];
-    if (r > 2) { T t = v[2]; if (r > 3) t += v[3]; s += t; }
-    if (r > 4) {
-        T t = v[4];
-        if (r > 5) t += v[5];
-        if (r > 6) { T q = v[6]; if (r > 7) q += v[7]; t += q; }
-        s += t;
+    switch (r) {
+        case 0: return T(0);
+        case 1: return v[0];
+        case 2: return v[0] + v[1];
+        case 3: return (v[0] + v[1]) + v[2];
+        case 4: return (v[0] + v[1]) + (v[2] + v[3]);
+        case 5: return ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
+        case 6: return ((v[0] + v[1]) + (v[2] + v[3])) + (v[4] + v[5]);
+        case 7: return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + v[6]);
+        default: return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
     }
-    return s;
+}
+
+// the same with edge weights, products and sums in one operation
+template <typename T>
+__device__ __forceinline__ T pass_dot(const T (&v)[8], const T (&w)[8], int r) {
+    auto two = [&](int u) { return fma(v[u + 1], w[u + 1], v[u] * w[u]); };
+    switch (r) {
+        case 0: return T(0);
+        case 1: return v[0] * w[0];
+        case 2: return two(0);
+        case 3: return fma(v[2], w[2], two(0));
+        case 4: return two(0) + two(2);
+        case 5: return fma(v[4], w[4], two(0) + two(2));
+        case 6: return (two(0) + two(2)) + two(4);
+        case 7: return (two(0) + two(2)) + fma(v[6], w[6], two(4));
+        default: return (two(0) + two(2)) + (two(4) + two(6));
+    }
 }
 
 template <typename T, class Epi>
@@ -683,46 +705,78 @@ __device__ __forceinline__ void slices_only_gather(const RowSched& S, const T* _
     const int gw = blockIdx.x * (int)(blockDim.x >> 5) + (threadIdx.x >> 5);
     const int nw = gridDim.x * (int)(blockDim.x >> 5);
     const T* __restrict__ sw = S.swts<T>();
-    int64_t o0 = 0, o1 = 0;
-    if (gw < S.n_slices) { o0 = S.sell_off[gw]; o1 = S.sell_off[gw + 1]; }
+    // [oa, ea): this slice, [ob, eb): the next, whose offsets are loaded a slice earlier; in: the first
+    // eight indices of this slice (-1 beyond its width)
+    int64_t oa = 0, ea = 0, ob = 0, eb = 0;
+    if (gw < S.n_slices) { oa = S.sell_off[gw]; ea = S.sell_off[gw + 1]; }
+    if (gw + nw < S.n_slices) { ob = S.sell_off[gw + nw]; eb = S.sell_off[gw + nw + 1]; }
+    int32_t in[8];
+    auto load_first = [&](int64_t o, int w) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) in[u] = u < w ? __ldcs(S.sell_ci + o + (int64_t)u * 32 + lane) : -1;
+    };
+    load_first(oa, (int)((ea - oa) >> 5));
     for (int s = gw; s < S.n_slices; s += nw) {
-        const int64_t oa = o0;
-        const int wa = (int)((o1 - o0) >> 5);
-        if (s + nw < S.n_slices) { o0 = S.sell_off[s + nw]; o1 = S.sell_off[s + nw + 1]; }   // next slice
+        const int wa = (int)((ea - oa) >> 5);
         const int64_t row = S.light0 + (int64_t)s * 32 + lane;
         const typename Epi::Pre pre = epi.pre(row);
+        int64_t oc = 0, ec = 0;
+        if (s + 2 * nw < S.n_slices) { oc = S.sell_off[s + 2 * nw]; ec = S.sell_off[s + 2 * nw + 1]; }
         T s0 = 0, s1 = 0;
-        for (int q = 0; q < wa; q += 8) {
-            int32_t ia[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) ia[u] = q + u < wa ? __ldcs(S.sell_ci + oa + (int64_t)(q + u) * 32 + lane) : -1;
-            T va[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) va[u] = ia[u] >= 0 ? __ldg(x + ia[u]) : T(0);
-            if (sw) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (sizeof(T) == 4 || q + u < wa)
-                        va[u] *= ia[u] >= 0 ? __ldcs(sw + oa + (int64_t)(q + u) * 32 + lane) : T(0);
-            }
+        auto add_pass = [&](const int32_t (&ia)[8], T (&va)[8], int q) {
             if constexpr (sizeof(T) == 4) {
+                if (sw) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) va[u] *= ia[u] >= 0 ? __ldcs(sw + oa + (int64_t)(q + u) * 32 + lane) : T(0);
+                }
                 s0 += (va[0] + va[1]) + (va[2] + va[3]);
                 s1 += (va[4] + va[5]) + (va[6] + va[7]);
             } else {
-                const T t = pass_sum(va, wa - q);
+                T t;
+                if (sw) {
+                    T wt[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) wt[u] = ia[u] >= 0 ? __ldcs(sw + oa + (int64_t)(q + u) * 32 + lane) : T(0);
+                    t = pass_dot(va, wt, wa - q);
+                } else {
+                    t = pass_sum(va, wa - q);
+                }
                 s0 = q == 0 ? t : s0 + t;
             }
+        };
+        {
+            T va[8];
+            int32_t ia[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ia[u] = in[u];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) va[u] = ia[u] >= 0 ? __ldg(x + ia[u]) : T(0);
+            load_first(ob, (int)((eb - ob) >> 5));
+            add_pass(ia, va, 0);
+        }
+        for (int q = 8; q < wa; q += 8) {
+            T va[8];
+            int32_t ia[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ia[u] = q + u < wa ? __ldcs(S.sell_ci + oa + (int64_t)(q + u) * 32 + lane) : -1;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) va[u] = ia[u] >= 0 ? __ldg(x + ia[u]) : T(0);
+            add_pass(ia, va, q);
         }
         if constexpr (sizeof(T) == 4) s0 += s1;
         if (row < S.n) epi.fin(row, pre, row == skip ? T(0) : s0);
+        oa = ob;
+        ea = eb;
+        ob = oc;
+        eb = ec;
     }
 }
 
 // The slices-only kernels are used when every row is sliced: relabelling on, sliced copy on, no
 // work items (light0 = 0, so the skipped row, too, is in a slice).
 __host__ __device__ inline bool slices_only(const RowSched& S) { return S.sell && S.n_items == 0; }
-// resident CTAs per SM of the plain sliced gathers (FP64 wants 40 registers)
-template <typename T> struct SliceBlocks { static constexpr int value = sizeof(T) == 4 ? 8 : 6; };
+// resident CTAs per SM of the plain sliced gathers (the indices held ahead want 40 and 64 registers)
+template <typename T> struct SliceBlocks { static constexpr int value = sizeof(T) == 4 ? 6 : 4; };
 
 // Epilogue of the plain gather: g[row] = sum over the row (0 for the skipped row).
 template <typename T>

@@ -391,11 +391,24 @@ __global__ void __launch_bounds__(ClThreads<T>::value, 1) k_minres_cluster(Inner
 #pragma unroll
                     for (int u = 0; u < 8; ++u) va[u] = ia[u] >= 0 ? __ldcg(zg + ia[u]) : T(0);
                 }
+                T t;
                 if (sw) {
+                    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) va[u] *= ia[u] >= 0 ? __ldg(sw + o0 + (int64_t)(q + u) * 32 + lane) : T(0);
+                        for (int u = 0; u < 8; ++u)
+                            va[u] *= ia[u] >= 0 ? __ldg(sw + o0 + (int64_t)(q + u) * 32 + lane) : T(0);
+                        t = cl_pass_sum(va, wa - q);
+                    } else {
+                        T wt[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            wt[u] = ia[u] >= 0 ? __ldg(sw + o0 + (int64_t)(q + u) * 32 + lane) : T(0);
+                        t = pass_dot(va, wt, wa - q);
+                    }
+                } else {
+                    t = cl_pass_sum(va, wa - q);
                 }
-                g0 = q == 0 ? cl_pass_sum(va, wa) : g0 + cl_pass_sum(va, wa - q);
+                g0 = q == 0 ? t : g0 + t;
             }
             const T z = zc[l];
             T y = Ad[l] * z - g0;

@@ -849,7 +849,7 @@ __device__ __forceinline__ void ml_phase1_finish(const InnerArgs<T>& a, T acc0, 
 
 // resident CTAs per SM of the kernels that do row arithmetic in a sliced gather: FP32 wants the warps in
 // flight; in FP64 every CTA's reduction costs FP64 issue slots (a warp sum as much as five rows)
-template <typename T> struct SlicedRows { static constexpr int ctas = sizeof(T) == 4 ? 5 : 3; };
+template <typename T> struct SlicedRows { static constexpr int ctas = sizeof(T) == 4 ? 4 : 3; };
 
 template <typename T, int NC>
 __global__ void __launch_bounds__(kThreads) k_ml_phase1(InnerArgs<T> a) {
