@@ -9,9 +9,7 @@
 //   rotate        X <- X S(:, a:b) in place, row tiles in shared memory (restart)
 //   true_residual ||L v_j - lambda_j v_j||                           (final check)
 //   setup         degrees, maximum degree and its vertex, row classes (Remark 4.1)
-// The tall-skinny kernels stage a tile of basis rows in shared memory once and use
-// it twice (row-wise update, column-wise dot products), so U and V are read once
-// per Gram-Schmidt pass.
+// The tall-skinny kernels give a thread whole rows and go over the columns in batches held in registers.
 #include <algorithm>
 #include <mutex>
 
@@ -743,108 +741,134 @@ void outer_arrow_eig(const double* H, int ldh, int k, int w, double* theta, doub
 
 // ------------------------------------------------------------------ tall-skinny passes (orthonormalisation, H column)
 
-constexpr int kTsRows = 64;              // rows per shared-memory tile
 constexpr int kTsMaxCols = kMMax + kCMax;
-constexpr int kTsColsPerWarp = (kTsMaxCols + kWarps - 1) / kWarps;
 
 // MODE 0: dots only:      out = [Q^T z, 1^T z, z^T z]
 // MODE 1: update + dots:  z <- z - Q h - mu 1, written back; out = [Q^T z, 1^T z]
 // MODE 2: update + norm:  as MODE 1, out = [z^T z]
 // Q = [U(:, 0:k) V(:, 0:c)].  coef = [h (k + c), mu].  The last block turns the sums
 // into the coefficients of the next pass (coef_next) or into the final norm.
+//
+// Bound by the FP64 pipe, one FMA lane per clock and SM as measured (an FP64 instruction whose predicate
+// is false costs as much as one whose predicate is true): n (k + c) FMAs per dot pass and per update.  So a
+// thread owns whole rows and nothing is done twice or under a predicate: the update is one FMA per column,
+// the dots go over the columns in batches of eight (then four, two, one) whose accumulators sit in
+// registers, and a batch is reduced once, at the end.  A row's columns are read again by the next
+// batches from L1 / L2.  Measured at n = 1.3 million, 15 columns: dots 66 us (62 us of FMAs); tiles of Q in
+// shared memory with a partial sum per tile and column took 94-107 us.
+constexpr int kTsBatch = 8;
+
+__device__ __forceinline__ const double* ts_col(const OuterArgs& a, int k, int j) {
+    return j < k ? a.U + (int64_t)j * a.ld : a.V + (int64_t)(j - k) * a.ld;
+}
+
+// sums over the block of NV per-thread values, into slots slot0 .. slot0 + NV - 1 of this block's partials
+template <int NV>
+__device__ __forceinline__ void ts_store(const OuterArgs& a, const double (&v)[NV], int slot0, double (*red)[kTsBatch]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+    double o[1];
+    warp_reduce_multi<double, NV>(v, o);
+    constexpr int G = 32 / NV;
+    if (lane % G == 0) red[warp][lane / G] = o[0];
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double s = red[0][threadIdx.x];
+        for (int w = 1; w < W; ++w) s += red[w][threadIdx.x];
+        a.partial[(size_t)(slot0 + threadIdx.x) * a.pstride + blockIdx.x] = s;
+    }
+    __syncthreads();
+}
+
+// Q(:, j0 : j0 + NB)^T z
+template <int NB>
+__device__ __forceinline__ void ts_dots(const OuterArgs& a, int k, int j0, const double* z, double (*red)[kTsBatch]) {
+    const double* col[NB];
+    double acc[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        col[i] = ts_col(a, k, j0 + i);
+        acc[i] = 0.0;
+    }
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll 2
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < a.n; r += step) {
+        const double zr = z[r];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) acc[i] += __ldg(col[i] + r) * zr;
+    }
+    ts_store<NB>(a, acc, j0, red);
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(kThreads) k_tall_skinny(OuterArgs a, int k, int c, const double* z_in,
                                                           double* z_out, const double* coef, double* coef_next,
                                                           double* Hcol, int hcol) {
-    extern __shared__ double tsm[];
     const int nq = k + c;
-    double* Qs = tsm;                           // [nq][kTsRows]
-    double* zs = tsm + (size_t)nq * kTsRows;    // [kTsRows]
-    double* hs = zs + kTsRows;                  // [nq + 1]
+    __shared__ double hs[kTsMaxCols + 1];
     __shared__ double red[kTsMaxCols + 2];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (MODE != 0)
+    __shared__ double wred[kWarps][kTsBatch];
+    const int tid = threadIdx.x;
+    if (MODE != 0) {
         for (int j = tid; j <= nq; j += blockDim.x) hs[j] = coef[j];
+        __syncthreads();
+    }
     const int nv = (MODE == 0) ? nq + 2 : (MODE == 1 ? nq + 1 : 1);
-    double acc[kTsColsPerWarp + 2];
-#pragma unroll
-    for (int i = 0; i < kTsColsPerWarp + 2; ++i) acc[i] = 0.0;
-    for (int64_t r0 = (int64_t)blockIdx.x * kTsRows; r0 < a.n; r0 += (int64_t)gridDim.x * kTsRows) {
-        __syncthreads();
-        for (int idx = tid; idx < nq * kTsRows; idx += blockDim.x) {
-            const int j = idx / kTsRows, rr = idx % kTsRows;
-            const int64_t r = r0 + rr;
-            const double* col = j < k ? a.U + (int64_t)j * a.ld : a.V + (int64_t)(j - k) * a.ld;
-            Qs[idx] = r < a.n ? col[r] : 0.0;
-        }
-        for (int rr = tid; rr < kTsRows; rr += blockDim.x) {
-            const int64_t r = r0 + rr;
-            zs[rr] = r < a.n ? z_in[r] : 0.0;
-        }
-        __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t rb = (int64_t)blockIdx.x * blockDim.x + tid;
+    double s1 = 0.0, s2 = 0.0;                             // 1^T z, z^T z
+    for (int64_t r = rb; r < a.n; r += step) {
+        double z = z_in[r];
         if (MODE != 0) {
-            // four threads per row split the columns, then combine with shuffles
-            const int rr = tid >> 2, part = tid & 3;
-            double s = 0.0;
-            for (int j = part; j < nq; j += 4) s += Qs[j * kTsRows + rr] * hs[j];
-            s += __shfl_xor_sync(kFull, s, 1);
-            s += __shfl_xor_sync(kFull, s, 2);
-            __syncthreads();
-            if (part == 0) {
-                const int64_t r = r0 + rr;
-                const double zn = (r < a.n) ? zs[rr] - s - hs[nq] : 0.0;
-                zs[rr] = zn;
-                if (r < a.n) z_out[r] = zn;
+            double q0 = 0.0, q1 = 0.0;
+            int j = 0;
+#pragma unroll 2
+            for (; j + 4 <= nq; j += 4) {
+                const double v0 = __ldg(ts_col(a, k, j) + r), v1 = __ldg(ts_col(a, k, j + 1) + r);
+                const double v2 = __ldg(ts_col(a, k, j + 2) + r), v3 = __ldg(ts_col(a, k, j + 3) + r);
+                q0 += v0 * hs[j];
+                q1 += v1 * hs[j + 1];
+                q0 += v2 * hs[j + 2];
+                q1 += v3 * hs[j + 3];
             }
-            __syncthreads();
+            for (; j < nq; ++j) q0 += __ldg(ts_col(a, k, j) + r) * hs[j];
+            z = z - (q0 + q1) - hs[nq];
+            z_out[r] = z;
         }
-        if (MODE == 2) {
-            for (int rr = tid; rr < kTsRows; rr += blockDim.x) acc[0] += zs[rr] * zs[rr];
-        } else {
-#pragma unroll
-            for (int i = 0; i < kTsColsPerWarp; ++i) {
-                const int j = warp + i * kWarps;
-                if (j < nq) {
-                    double s = 0.0;
-                    for (int rr = lane; rr < kTsRows; rr += 32) s += Qs[j * kTsRows + rr] * zs[rr];
-                    acc[i] += s;
-                }
-            }
-            if (warp == 0)
-                for (int rr = lane; rr < kTsRows; rr += 32) acc[kTsColsPerWarp] += zs[rr];
-            if (MODE == 0 && warp == 1)
-                for (int rr = lane; rr < kTsRows; rr += 32) acc[kTsColsPerWarp + 1] += zs[rr] * zs[rr];
-        }
+        if (MODE != 2) s1 += z;
+        if (MODE != 1) s2 += z * z;
     }
-    // gather the per-warp column sums into a per-thread vector of nv slots, then reduce
-    __shared__ double bsum[kTsMaxCols + 2];
-    __syncthreads();
-    if (MODE == 2) {
-        double v = block_sum0(acc[0]);
-        if (tid == 0) bsum[0] = v;
+    if (MODE != 2) {
+        const double* z = MODE == 0 ? z_in : z_out;        // a thread reads the rows that it wrote
+        int j = 0;
+        for (; j + kTsBatch <= nq; j += kTsBatch) ts_dots<kTsBatch>(a, k, j, z, wred);
+        if (nq - j >= 4) { ts_dots<4>(a, k, j, z, wred); j += 4; }
+        if (nq - j >= 2) { ts_dots<2>(a, k, j, z, wred); j += 2; }
+        if (nq - j >= 1) ts_dots<1>(a, k, j, z, wred);
+    }
+    if (MODE == 0) {
+        const double v[2] = {s1, s2};
+        ts_store<2>(a, v, nq, wred);
     } else {
-#pragma unroll
-        for (int i = 0; i < kTsColsPerWarp; ++i) {
-            const int j = warp + i * kWarps;
-            double v = warp_sum(acc[i]);
-            if (lane == 0 && j < nq) bsum[j] = v;
-        }
-        double v = warp_sum(acc[kTsColsPerWarp]);
-        if (warp == 0 && lane == 0) bsum[nq] = v;
-        if (MODE == 0) {
-            double w = warp_sum(acc[kTsColsPerWarp + 1]);
-            if (warp == 1 && lane == 0) bsum[nq + 1] = w;
-        }
+        const double v[1] = {MODE == 1 ? s1 : s2};
+        ts_store<1>(a, v, MODE == 1 ? nq : 0, wred);
     }
-    __syncthreads();
-    for (int i = tid; i < nv; i += blockDim.x) a.partial[(size_t)i * a.pstride + blockIdx.x] = bsum[i];
     __threadfence();
     __syncthreads();
     __shared__ int last;
     if (tid == 0) last = (atomicAdd(a.counter, 1u) == gridDim.x - 1);
     __syncthreads();
     if (!last) return;
-    last_block_sum(a.partial, a.pstride, gridDim.x, nv, red, a.counter);
+    {
+        const int lane = tid & 31, W = blockDim.x >> 5;
+        for (int i = tid >> 5; i < nv; i += W) {
+            double s = 0.0;
+            for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(a.partial + (size_t)i * a.pstride + b);
+            s = warp_sum(s);
+            if (lane == 0) red[i] = s;
+        }
+        if (tid == 0) *a.counter = 0u;
+        __syncthreads();
+    }
     const double inv_n = 1.0 / (double)a.n;
     if (MODE == 0 && Hcol != nullptr) {
         // H(0:nq, hcol) and the symmetric row from the dots U^T w
@@ -871,16 +895,6 @@ __global__ void __launch_bounds__(kThreads) k_tall_skinny(OuterArgs a, int k, in
     }
 }
 
-static void ts_smem_attr() {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        const int bytes = (int)(sizeof(double) * ((size_t)kTsMaxCols * kTsRows + kTsRows + kTsMaxCols + 1));
-        cudaFuncSetAttribute(k_tall_skinny<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        cudaFuncSetAttribute(k_tall_skinny<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        cudaFuncSetAttribute(k_tall_skinny<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    });
-}
-
 // One launch wave: at most SMs x resident CTAs (registers and dynamic shared memory decide the
 // latter), so a tile loop never runs as a full wave plus a partial one.
 static int wave_of(const void* fn, size_t smem, int want) {
@@ -898,20 +912,24 @@ static int wave_of(const void* fn, size_t smem, int want) {
     return want < cap ? want : cap;
 }
 
-static size_t ts_smem(int nq) { return sizeof(double) * ((size_t)nq * kTsRows + kTsRows + nq + 1); }
+// Two CTAs of 256 threads per SM keep the FP64 pipe and enough loads busy; small graphs take CTAs of 64
+// rows, so that every SM has some.
+template <int MODE>
+static void tall_skinny(const OuterArgs& a, int k, int c, const double* z_in, double* z_out, const double* coef,
+                        double* coef_next, double* Hcol, int hcol, cudaStream_t s) {
+    constexpr int kSms = 152;
+    const int threads = a.n < (int64_t)kSms * kThreads ? 64 : kThreads;
+    const int grid = (int)std::min<int64_t>((a.n + threads - 1) / threads, threads == 64 ? 4 * kSms : 2 * kSms);
+    k_tall_skinny<MODE><<<std::min(grid, a.ts_blocks), threads, 0, s>>>(a, k, c, z_in, z_out, coef, coef_next, Hcol,
+                                                                       hcol);
+}
 
 void outer_cgs2(const OuterArgs& a, int k, int c, cudaStream_t s) {
-    ts_smem_attr();
-    const int nq = k + c;
     double* cA = a.dscratch + 8;                 // coefficients of pass B
     double* cB = a.dscratch + 8 + kTsMaxCols + 1; // coefficients of pass C
-    const size_t sm = ts_smem(nq);
-    k_tall_skinny<0><<<wave_of((const void*)k_tall_skinny<0>, sm, a.ts_blocks), kThreads, sm, s>>>(
-        a, k, c, a.Z, nullptr, nullptr, cA, nullptr, 0);
-    k_tall_skinny<1><<<wave_of((const void*)k_tall_skinny<1>, sm, a.ts_blocks), kThreads, sm, s>>>(
-        a, k, c, a.Z, a.Z, cA, cB, nullptr, 0);
-    k_tall_skinny<2><<<wave_of((const void*)k_tall_skinny<2>, sm, a.ts_blocks), kThreads, sm, s>>>(
-        a, k, c, a.Z, a.Z, cB, nullptr, nullptr, 0);
+    tall_skinny<0>(a, k, c, a.Z, nullptr, nullptr, cA, nullptr, 0, s);
+    tall_skinny<1>(a, k, c, a.Z, a.Z, cA, cB, nullptr, 0, s);
+    tall_skinny<2>(a, k, c, a.Z, a.Z, cB, nullptr, nullptr, 0, s);
 }
 
 // ------------------------------------------------------------------ back-map of a single inner solve
@@ -1017,13 +1035,10 @@ int gather_ctas_per_sm(int tpb, int hub_bytes) {
 }
 
 void outer_expand(const OuterArgs& a, int k, int lanes, cudaStream_t s) {
-    ts_smem_attr();
     outer_gather(a, a.Z, lanes, s);
     k_expand_rows<<<a.ew_blocks, kThreads, 0, s>>>(a, k);
     // H(0:k+1, k) = U(:, 0:k+1)^T W(:, k)
-    k_tall_skinny<0><<<wave_of((const void*)k_tall_skinny<0>, ts_smem(k + 1), a.ts_blocks), kThreads,
-                       ts_smem(k + 1), s>>>(a, k + 1, 0, a.W + (int64_t)k * a.ld, nullptr,
-                                                                   nullptr, nullptr, a.H, k);
+    tall_skinny<0>(a, k + 1, 0, a.W + (int64_t)k * a.ld, nullptr, nullptr, nullptr, a.H, k, s);
 }
 
 void outer_laplacian(const OuterArgs& a, const double* x, double* y, int lanes, cudaStream_t s) {
