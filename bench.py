@@ -311,6 +311,18 @@ def kernel_bytes(kind, n, Z, c, word, n_long=None, n_slices=None, ml=None):
         struct = 8 * (n + 1) if not n_slices else 8 * (n_long + 1) + 8 * (n_slices + 1)
         return ((25 + 4 * c) * word * n + 8 * n + 2 * (struct + 4 * Z)
                 + 2 * (4 + word) * nnz_c + (16 + 5 * word) * n_c)
+    if kind == "gather_ml_s":
+        # graphs whose rows are all sliced: gather and rows in one kernel (no neighbour sums stored or read)
+        return (kernel_bytes("gather", n, Z, c, word, n_long, n_slices)
+                + kernel_bytes("rows_ml", n, Z, c, word) - 2 * word * n)
+    if kind == "phase2_ml_s":
+        # the same graphs: the residual is formed in the gather of x0 (b read there, not in the restriction),
+        # the gather of x1 does the post-smoothing and phase 2b (no W x1 stored or read), and a coarse level
+        # moves b, D^{-1} b, x1 and its diagonal once more than the per-entry form
+        n_c, nnz_c = ml
+        struct = 8 * (n + 1) if not n_slices else 8 * (n_long + 1) + 8 * (n_slices + 1)
+        return ((21 + 4 * c) * word * n + 8 * n + 2 * (struct + 4 * Z)
+                + 2 * (4 + word) * nnz_c + (16 + 9 * word) * n_c)
     if kind == "gather":
         struct = 8 * (n + 1) if not n_slices else 8 * (n_long + 1) + 8 * (n_slices + 1)
         return struct + 4 * Z + 2 * word * n
@@ -324,11 +336,12 @@ def kernel_bytes(kind, n, Z, c, word, n_long=None, n_slices=None, ml=None):
 KERNEL_NAMES = {"gather": "k_phase1_gather (trimmed-operator SpMV gather)",
                 "rows": "k_phase1 (operator row epilogue + MINRES update)",
                 "phase2": "k_phase2 (SMW preconditioner + MINRES reductions)"}
-KERNEL_NAMES_ML = {"gather": "k_phase1_gather (trimmed-operator SpMV gather)",
-                   "rows": "k_ml_phase1 (operator row epilogue + MINRES update)",
-                   "phase2": "multilevel phase 2 (13 launches on the 128^3 grid in FP32): ml_phase2a, ml_project, "
-                             "one V-cycle (two level-0 gathers, restriction, prolongation, fused coarse-level "
-                             "sweeps), ml_phase2b with the level-0 post-smoothing, ml_phase2c"}
+KERNEL_NAMES_ML = {"gather": "k_ml_phase1_s (trimmed-operator SpMV gather with the row epilogue and the MINRES "
+                             "update; k_phase1_gather where rows are not all sliced)",
+                   "rows": "k_ml_phase1 (operator row epilogue + MINRES update, where not part of the gather)",
+                   "phase2": "multilevel phase 2: ml_phase2a, ml_project, one V-cycle (two level-0 gathers, "
+                             "restriction, prolongation, one sweep down and up per coarse level), the level-0 "
+                             "post-smoothing with phase 2b, ml_phase2c"}
 STAT_OF = {"gather": "inner_phase1_ms", "rows": "inner_rows_ms", "phase2": "inner_phase2_ms"}
 
 GATHER_SOURCES = ["paper_1710_07080_gb300/csrc/common.cuh", "paper_1710_07080_gb300/csrc/inner_impl.cuh"]
@@ -383,6 +396,9 @@ def kernel_rooflines(st, n, Z, word, workload, prec_tag):
         ms = st[STAT_OF[kind]]
         avg_s = ms / 1e3 / max(1, nl)
         bkind = kind + "_ml" if ml and kind != "gather" else kind
+        if ml and n_slices and not st["n_long_rows"]:
+            # every row sliced: phase 1 is one kernel, timed as the gather
+            bkind = {"gather": "gather_ml_s", "phase2": "phase2_ml_s"}.get(kind, bkind)
         b = kernel_bytes(bkind, n, Z, c_avg, word, st["n_long_rows"], n_slices,
                          (st.get("ml_coarse_n", 0), st.get("ml_coarse_nnz", 0)))
         ach = b / avg_s / 1e9 if avg_s > 0 else None

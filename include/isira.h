@@ -142,7 +142,8 @@ typedef struct {
     long long spmv_launches;  /* launches of the inner operator's gather kernel (phase 1) */
     double solve_ms;          /* host wall time of the last isira_solve */
     double inner_phase1_ms;   /* summed device time of the phase-1 gather launches (profiling on only); in the
-                                 one-launch solve of a small graph, of its gather and row arithmetic */
+                                 one-launch solve of a small graph, and with the multilevel preconditioner on
+                                 graphs whose rows are all sliced, of gather and row arithmetic together */
     long long inner_phase1_timed; /* number of phase-1 gather launches timed */
     long long inner_phase1_csum;  /* sum of the deflation rank c over the timed phase-1 launches */
     long long kernel_launches;    /* kernels launched by the last isira_solve */
@@ -278,8 +279,8 @@ ISIRA_API isira_status isira_residual_history(isira_handle h, double* h_rnorm, i
  * Output as isira_sym_eig (d_theta ascending, d_S overwritten by the k eigenvectors, sign rule).
  * If Q0^T H0 Q0 is not diagonal to a few rounding errors the arrowhead path refuses and parallel
  * Jacobi (isira_sym_eig, warm-started from Q0) produces the result instead; *path (may be NULL)
- * receives 1 for the arrowhead path, 0 for Jacobi.  Allocates a small device scratch and
- * synchronises the stream. */
+ * receives 1 for the arrowhead path, 0 for Jacobi.  Takes a small device scratch (allocated on the first
+ * calls, at most 16 of 36 KB kept by the process for later ones) and synchronises the stream. */
 ISIRA_API isira_status isira_sym_eig_warm(int k, int warm_w, const double* d_H, double* d_theta, double* d_S,
                                           int* path, void* stream);
 

@@ -372,7 +372,7 @@ def sym_eig(H):
         raise ValueError("H must be a square matrix of order 1..64")
     _check_tensor(H.contiguous(), "H", (torch.float64,), (H.shape[0], H.shape[0]))   # includes the device
     k = H.shape[0]
-    Hc = H.t().contiguous()          # column-major
+    Hc = H.contiguous()              # the library takes (H + H^T) / 2, so rows serve as columns
     th = torch.empty(k, dtype=torch.float64, device=H.device)
     S = torch.empty((k, k), dtype=torch.float64, device=H.device)
     check(lib.isira_sym_eig(k, _ptr(Hc), _ptr(th), _ptr(S), _stream_ptr()), "isira_sym_eig")
@@ -393,9 +393,9 @@ def sym_eig_warm(H, S0):
     _check_tensor(S0.contiguous(), "S0", (torch.float64,), tuple(S0.shape))
     _check_cuda(H=H, S0=S0)
     w = S0.shape[0]
-    Hc = H.t().contiguous()
-    S = torch.zeros((k, k), dtype=torch.float64, device=H.device)
-    S[:w, :w] = S0.t()                    # column-major, ld k
+    Hc = H.contiguous()                   # the library takes (H + H^T) / 2, so rows serve as columns
+    S = torch.empty((k, k), dtype=torch.float64, device=H.device)
+    S[:w, :w] = S0.t()                    # column-major, ld k; the call reads this block and writes all of S
     th = torch.empty(k, dtype=torch.float64, device=H.device)
     path = C.c_int(-1)
     check(lib.isira_sym_eig_warm(k, w, _ptr(Hc), _ptr(th), _ptr(S), C.byref(path), _stream_ptr()),

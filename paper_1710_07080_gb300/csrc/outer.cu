@@ -322,9 +322,8 @@ void outer_sym_eig(const double* H, int ldh, int k, double* theta, double* S, in
 //   setup    one CTA per column i of Q0: one Newton-Schulz step q~_i = q_i (3/2) - Q0 Q0^T q_i / 2
 //            (keeps the warm-start basis orthonormal over many steps), d_i = q~_i^T H0 q~_i,
 //            z_i = q~_i^T h, and the largest |q_j^T H0 q~_i|, j != i; the last CTA deflates;
-//   roots    one warp per root: safeguarded Newton, in coordinates centred on the nearer pole d_o,
-//            on f(lambda) times the interval's end poles, from the root of a one-pole model,
-//            bisection when a step leaves the bracket;
+//   roots    one warp per root: safeguarded rational interpolation, in coordinates centred on the nearer
+//            pole d_o, with both end poles of the interval, bisection when a step leaves the bracket;
 //   zhat     one warp per undeflated pole (Loewner's formula as a product of bounded ratios);
 //   vectors  one CTA per eigenpair: the vector in the arrowhead basis, its place in ascending
 //            order, S(:, place) = Q~ x with the sign rule of outer_sym_eig.
@@ -333,7 +332,8 @@ void outer_sym_eig(const double* H, int ldh, int k, double* theta, double* S, in
 
 constexpr double kEpsD = 2.220446049250313e-16;   // unit roundoff x 2 (machine epsilon, binary64)
 constexpr int kArrowThreads = 64;                 // >= kMMax: one thread per row of H
-constexpr int kArrowMaxIt = 200;                  // iteration limit of one root (Newton ends in 3-15; the
+constexpr int kArrowSetup = 4 * kArrowThreads;    // setup: four threads share a row's products
+constexpr int kArrowMaxIt = 200;                  // iteration limit of one root (a few model steps; the
                                                   // bracket test ends a run of bisection steps)
 constexpr int kArrowLd = kMMax + 1;
 
@@ -355,6 +355,7 @@ __device__ void arrow_deflate(int k, int w, ArrowWork* aw, HostStatus* hs, doubl
     __shared__ int ord[kMMax];
     __shared__ double rm[3][kArrowThreads / 32];
     __shared__ int refused, nrot_s;
+    __shared__ double ds[kMMax], zs[kMMax];               // d and |z| in ascending order of d
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
     const bool arrow = w < k;
     double dv = 0.0, zv = 0.0, ov = 0.0;
@@ -369,7 +370,7 @@ __device__ void arrow_deflate(int k, int w, ArrowWork* aw, HostStatus* hs, doubl
     double a = warp_max(fmax(fabs(dv), fabs(zv)));
     double o = warp_max(ov);
     double zq = warp_sum(zv * zv);
-    if (lane == 0) { rm[0][wp] = a; rm[1][wp] = o; rm[2][wp] = zq; }
+    if (lane == 0 && wp < kArrowThreads / 32) { rm[0][wp] = a; rm[1][wp] = o; rm[2][wp] = zq; }
     __syncthreads();
     const double scale = fmax(fmax(rm[0][0], rm[0][1]), fabs(alpha));
     const double offmax = fmax(rm[1][0], rm[1][1]);
@@ -387,10 +388,19 @@ __device__ void arrow_deflate(int k, int w, ArrowWork* aw, HostStatus* hs, doubl
         int r = 0;
         for (int j = 0; j < w; ++j) r += (d[j] < dv) || (d[j] == dv && j < tid);
         ord[r] = tid;
+        ds[r] = dv;
+        zs[r] = fabs(zv);
     }
     __syncthreads();
+    const double tol = 8.0 * kEpsD * scale;
+    // the usual case, decided in parallel: nothing deflates
+    const bool plain = tid >= w || (zs[tid] > tol && (tid == 0 || ds[tid] - ds[tid - 1] > tol));
+    if (__syncthreads_and(arrow && plain)) {
+        if (tid < w) aw->pole[tid] = ord[tid];
+        if (tid == 0) { aw->m = w; aw->nd = 0; aw->nrot = 0; }
+        return;
+    }
     if (tid == 0) {
-        const double tol = 8.0 * kEpsD * scale;
         int m = 0, nd = 0, nrot = 0, last = -1;
         for (int r = 0; r < w; ++r) {
             const int i = ord[r];
@@ -439,67 +449,76 @@ __device__ void arrow_deflate(int k, int w, ArrowWork* aw, HostStatus* hs, doubl
     }
 }
 
-__global__ void __launch_bounds__(kArrowThreads) k_arrow_setup(const double* H, int ldh, int k, int w,
-                                                            const double* S, int lds, ArrowWork* aw,
-                                                            HostStatus* hs, double off_cap) {
+// Four threads share each product's terms (one thread per row ran five chains of w dependent FP64 FMAs
+// and loaded Q0 and H through 64 threads: 50.7 us at k = 41).
+__global__ void __launch_bounds__(kArrowSetup) k_arrow_setup(const double* H, int ldh, int k, int w, const double* S,
+                                                          int lds, ArrowWork* aw, HostStatus* hs, double off_cap) {
     extern __shared__ double arrow_sm[];
     double* Qs = arrow_sm;                    // Q0, ld kArrowLd
     double* Hs = arrow_sm + kMMax * kArrowLd; // H (symmetrised), ld kArrowLd
-    __shared__ double g[kMMax], qt[kMMax], t[kMMax];
+    __shared__ double g[kMMax], qt[kMMax], t[kMMax], of[kMMax];
     __shared__ double red[3][kArrowThreads / 32];
     __shared__ int is_last;
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, i = blockIdx.x;
-    for (int idx = tid; idx < w * w; idx += blockDim.x) {
-        const int r = idx % w, c = idx / w;
-        Qs[r + c * kArrowLd] = S[r + (int64_t)c * lds];
-    }
-    for (int idx = tid; idx < k * k; idx += blockDim.x) {
-        const int r = idx % k, c = idx / k;
-        Hs[r + c * kArrowLd] = H[r + (int64_t)c * ldh];
-    }
-    __syncthreads();
-    for (int idx = tid; idx < k * k; idx += blockDim.x) {
-        const int r = idx % k, c = idx / k;
-        if (r < c) {
-            const double v = 0.5 * (Hs[r + c * kArrowLd] + Hs[c + r * kArrowLd]);
-            Hs[r + c * kArrowLd] = v;
-            Hs[c + r * kArrowLd] = v;
+    for (int c = wp; c < k; c += kArrowSetup / 32)
+#pragma unroll
+        for (int u = 0; u < kMMax / 32; ++u) {
+            const int r = lane + 32 * u;
+            if (r < w && c < w) Qs[r + c * kArrowLd] = S[r + (int64_t)c * lds];
+            if (r < k) Hs[r + c * kArrowLd] = 0.5 * (H[r + (int64_t)c * ldh] + H[c + (int64_t)r * ldh]);
         }
-    }
-    if (tid < w) {                                        // g = Q0^T q_i
+    __syncthreads();
+    const int row = tid >> 2, part = tid & 3;
+    auto quad = [](double v) {
+        v += __shfl_xor_sync(kFull, v, 1);
+        return v + __shfl_xor_sync(kFull, v, 2);
+    };
+    {                                                     // g = Q0^T q_i
         double acc = 0.0;
-        for (int r = 0; r < w; ++r) acc += Qs[r + tid * kArrowLd] * Qs[r + i * kArrowLd];
-        g[tid] = acc;
+        if (row < w)
+            for (int r = part; r < w; r += 4) acc += Qs[r + row * kArrowLd] * Qs[r + i * kArrowLd];
+        acc = quad(acc);
+        if (part == 0) g[row] = acc;
     }
     __syncthreads();
-    if (tid < w) {                                        // q~_i = (3/2) q_i - (1/2) Q0 g
+    {                                                     // q~_i = (3/2) q_i - (1/2) Q0 g
         double acc = 0.0;
-        for (int j = 0; j < w; ++j) acc += Qs[tid + j * kArrowLd] * g[j];
-        qt[tid] = 1.5 * Qs[tid + i * kArrowLd] - 0.5 * acc;
+        if (row < w)
+            for (int j = part; j < w; j += 4) acc += Qs[row + j * kArrowLd] * g[j];
+        acc = quad(acc);
+        if (part == 0 && row < w) qt[row] = 1.5 * Qs[row + i * kArrowLd] - 0.5 * acc;
     }
     __syncthreads();
-    if (tid < w) {                                        // t = H0 q~_i
+    {                                                     // t = H0 q~_i
         double acc = 0.0;
-        for (int c = 0; c < w; ++c) acc += Hs[tid + c * kArrowLd] * qt[c];
-        t[tid] = acc;
+        if (row < w)
+            for (int c = part; c < w; c += 4) acc += Hs[row + c * kArrowLd] * qt[c];
+        acc = quad(acc);
+        if (part == 0) t[row] = acc;
     }
     __syncthreads();
-    double dd = 0.0, zz = 0.0, off = 0.0;
-    if (tid < w) {
-        dd = qt[tid] * t[tid];
-        if (w < k) zz = qt[tid] * Hs[tid + w * kArrowLd];
-        if (tid != i) {
-            double acc = 0.0;
-            for (int r = 0; r < w; ++r) acc += Qs[r + tid * kArrowLd] * t[r];
-            off = fabs(acc);
+    {                                                     // off-diagonal entries q_j^T t
+        double acc = 0.0;
+        if (row < w && row != i)
+            for (int r = part; r < w; r += 4) acc += Qs[r + row * kArrowLd] * t[r];
+        acc = quad(acc);
+        if (part == 0) of[row] = fabs(acc);
+    }
+    __syncthreads();
+    if (tid < kArrowThreads) {
+        double dd = 0.0, zz = 0.0, off = 0.0;
+        if (tid < w) {
+            dd = qt[tid] * t[tid];
+            if (w < k) zz = qt[tid] * Hs[tid + w * kArrowLd];
+            off = of[tid];
         }
+        dd = warp_sum(dd);
+        zz = warp_sum(zz);
+        off = warp_max(off);
+        if (lane == 0) { red[0][wp] = dd; red[1][wp] = zz; red[2][wp] = off; }
+        if (tid < k) aw->Q[tid + i * kMMax] = tid < w ? qt[tid] : 0.0;
+        if (i == 0 && w < k && tid < k) aw->Q[tid + w * kMMax] = tid == w ? 1.0 : 0.0;
     }
-    dd = warp_sum(dd);
-    zz = warp_sum(zz);
-    off = warp_max(off);
-    if (lane == 0) { red[0][wp] = dd; red[1][wp] = zz; red[2][wp] = off; }
-    if (tid < k) aw->Q[tid + i * kMMax] = tid < w ? qt[tid] : 0.0;
-    if (i == 0 && w < k && tid < k) aw->Q[tid + w * kMMax] = tid == w ? 1.0 : 0.0;
     __syncthreads();
     if (tid == 0) {
         aw->d[i] = red[0][0] + red[0][1];
@@ -521,12 +540,17 @@ __global__ void __launch_bounds__(kArrowThreads) k_arrow_setup(const double* H, 
 // two outer intervals) and mu = lambda - d_o:
 //   g(mu) = (alpha - d_o) - mu - S1(mu) + zeta_o / mu - zeta_f / (delta_f - mu),
 //   S1 = sum_{i != o, f} zeta_i / (delta_i - mu),  S2 = sum_{i != o, f} zeta_i / (delta_i - mu)^2,
-// zeta_i = z_i^2, delta_i = d_i - d_o.  Newton runs on F = (-mu)(delta_f - mu) g (h = -mu g without f),
-// which has no pole inside the interval:
-//   F = q r + zeta_o (mu - delta_f) + zeta_f mu,  q = mu^2 - delta_f mu,  r = (alpha - d_o) - mu - S1,
-//   F' = (2 mu - delta_f) r - q (1 + S2) + zeta_o + zeta_f.
-// g decreases through the root, so its sign keeps a bracket; steps that leave it are replaced by
-// bisection.
+// zeta_i = z_i^2, delta_i = d_i - d_o.  A step solves the rational model that has g's value and slope at mu
+// and both end poles (R.-C. Li, LAPACK Working Note 89, 1994): the near pole with its own weight, the far
+// pole with the weight q delta, delta = delta_f - mu, q = delta (1 + S2 + zeta_f / delta^2), that takes up
+// the slope of the rest; beyond the end poles the rest is linear.  In the correction eta both are
+// quadratics A eta^2 + B eta + C = 0:
+//   interior  A = zeta_o / mu - q - g, B = g (delta - mu) - delta zeta_o / mu - q mu, C = g mu delta,
+//   outer     A = -(1 + S2),           B = g - (1 + S2) mu - zeta_o / mu,             C = g mu.
+// It converges in a few steps from anywhere in the interval, where Newton on g times its poles took up
+// to 14 (33 us at k = 41).  g decreases through the root, so its sign keeps a bracket; steps that leave
+// it are replaced by bisection.  The start of an interior root solves the same model from the sums at
+// the interval's midpoint, which the choice of o needs anyway.
 __global__ void __launch_bounds__(32) k_arrow_roots(ArrowWork* aw) {
     if (aw->status) return;
     const int m = aw->m, j = blockIdx.x, lane = threadIdx.x;
@@ -559,7 +583,7 @@ __global__ void __launch_bounds__(32) k_arrow_roots(ArrowWork* aw) {
         s2 = warp_sum(a2);
     };
     int o;
-    double a, b;                                          // bracket of mu (endpoint 0 = the pole itself)
+    double a, b, mu = 0.0;                                // bracket of mu (endpoint 0 = the pole itself)
     if (j == 0) {
         o = 0;
         const double po = pole_at(0);
@@ -571,54 +595,119 @@ __global__ void __launch_bounds__(32) k_arrow_roots(ArrowWork* aw) {
         a = 0.0;
         b = fmax(0.0, alpha - po) + 1.0625 * aw->znorm;
     } else {
-        const double pl = pole_at(j - 1), pr = pole_at(j);
-        const double half = 0.5 * (pr - pl);
+        const double pl = pole_at(j - 1), pr = pole_at(j), d = pr - pl;
+        const double half = 0.5 * d, zl = zeta_at(j - 1), zr = zeta_at(j);
         double s1, s2;
-        sums(j - 1, -1, pl, half, s1, s2);
-        const double gm = (alpha - pl) - half - s1 + zeta_at(j - 1) / half;
-        if (gm > 0.0) { o = j; a = -half; b = 0.0; }      // root in (midpoint, p_j): centre on p_j
-        else { o = j - 1; a = 0.0; b = half; }            // root in (p_{j-1}, midpoint]
+        sums(j - 1, j, pl, half, s1, s2);
+        const double cm = (alpha - pl) - half - s1;       // g at the midpoint without the end poles
+        if (cm + (zl - zr) / half > 0.0) {                // root in (midpoint, p_j): centre on p_j
+            o = j; a = -half; b = 0.0;
+            const double bb = cm * d + zl + zr;
+            mu = -2.0 * zr * d / (bb + sqrt(fmax(bb * bb - 4.0 * cm * zr * d, 0.0)));
+        } else {                                          // root in (p_{j-1}, midpoint]
+            o = j - 1; a = 0.0; b = half;
+            const double bb = cm * d - zl - zr;
+            mu = 2.0 * zl * d / (sqrt(fmax(bb * bb + 4.0 * cm * zl * d, 0.0)) - bb);
+        }
     }
     const double po = pole_at(o), ao = alpha - po, zo = zeta_at(o);
-    // interior intervals: f is the other end pole; Newton runs on F = (-mu)(delta_f - mu) g(mu), which
-    // has neither pole of the interval; the outer intervals use h = -mu g(mu)
     const int f = (j > 0 && j < m) ? (o == j - 1 ? j : j - 1) : -1;
     const double df = f >= 0 ? pole_at(f) - po : 0.0, zf = f >= 0 ? zeta_at(f) : 0.0;
-    // start at the root of the model with the other poles' sum frozen at mu = 0:
-    // mu^2 - C mu - zeta_o = 0, C = (alpha - d_o) - S1(0) (- zeta_f / delta_f), taken on the bracket's side
-    double mu;
-    {
+    if (f < 0) {
+        // outer intervals start at the root of the model with the other poles' sum frozen at mu = 0:
+        // mu^2 - C mu - zeta_o = 0, C = (alpha - d_o) - S1(0), taken on the bracket's side
         double s1, s2;
         sums(o, f, po, 0.0, s1, s2);
-        const double cc = ao - s1 - (f >= 0 ? zf / df : 0.0), sq = sqrt(cc * cc + 4.0 * zo);
+        const double cc = ao - s1, sq = sqrt(cc * cc + 4.0 * zo);
         if (b == 0.0) mu = cc <= 0.0 ? 0.5 * (cc - sq) : -2.0 * zo / (cc + sq);
         else mu = cc >= 0.0 ? 0.5 * (cc + sq) : 2.0 * zo / (sq - cc);
-        if (!(mu > a && mu < b)) mu = 0.5 * (a + b);
+    }
+    if (!(mu > a && mu < b)) mu = 0.5 * (a + b);
+    // the same steps in FP32 first: they only have to bring the start close (a dozen FP64 operations in a row
+    // take a microsecond here), and what they end with is taken only inside the FP64 bracket
+    {
+        const float q0 = (float)(p0 - po), q1 = (float)(p1 - po), fz0 = (float)zeta0, fz1 = (float)zeta1;
+        const bool in0 = i0 < m && i0 != o && i0 != f, in1 = i1 < m && i1 != o && i1 != f;
+        const float fao = (float)ao, fzo = (float)zo, fzf = (float)zf, fdf = (float)df;
+        float fa = (float)a, fb = (float)b, fm = (float)mu;
+        for (int it = 0; it < 20; ++it) {
+            float t1 = 0.0f, t2 = 0.0f;
+            if (in0) {
+                const float inv = 1.0f / (q0 - fm), q = fz0 * inv;
+                t1 += q;
+                t2 += q * inv;
+            }
+            if (in1) {
+                const float inv = 1.0f / (q1 - fm), q = fz1 * inv;
+                t1 += q;
+                t2 += q * inv;
+            }
+            t1 = warp_sum(t1);
+            t2 = warp_sum(t2);
+            const float p = fzo / fm, dl = fdf - fm, ff = f >= 0 ? fzf / dl : 0.0f;
+            const float gv = fao - fm - t1 + p - ff;
+            if (gv > 0.0f) fa = fm;
+            else if (gv < 0.0f) fb = fm;
+            else break;                                   // zero, or not a number
+            float A, B, C;
+            if (f >= 0) {
+                const float q = dl * (1.0f + t2) + ff;
+                A = p - q - gv;
+                B = gv * (dl - fm) - p * dl - q * fm;
+                C = gv * fm * dl;
+            } else {
+                A = -(1.0f + t2);
+                B = gv + A * fm - p;
+                C = gv * fm;
+            }
+            const float eta = -2.0f * C / (B + copysignf(sqrtf(fmaxf(B * B - 4.0f * A * C, 0.0f)), B));
+            const float nw = fm + eta;
+            if (nw > fa && nw < fb) {
+                fm = nw;
+                if (fabsf(eta) <= 1e-6f * fabsf(fm)) break;
+            } else {
+                const float gm = fa * fb > 0.0f ? copysignf(sqrtf(fabsf(fa)) * sqrtf(fabsf(fb)), fa) : 0.0f;
+                fm = gm > fa && gm < fb ? gm : 0.5f * (fa + fb);
+            }
+        }
+        if ((double)fm > a && (double)fm < b) mu = (double)fm;
     }
     for (int it = 0; it < kArrowMaxIt; ++it) {
         double s1, s2;
         sums(o, f, po, mu, s1, s2);
-        double gv, F, Fp;
-        if (f >= 0) {
-            gv = ao - mu - s1 + zo / mu - zf / (df - mu);
-            const double q = mu * mu - df * mu, r = ao - mu - s1;
-            F = q * r + zo * (mu - df) + zf * mu;
-            Fp = (2.0 * mu - df) * r - q * (1.0 + s2) + zo + zf;
-        } else {
-            gv = ao - mu - s1 + zo / mu;
-            F = -mu * ao + mu * mu + mu * s1 - zo;
-            Fp = -ao + 2.0 * mu + s1 + mu * s2;
-        }
+        const double p = zo / mu, dl = df - mu, ff = f >= 0 ? zf / dl : 0.0;
+        const double gv = ao - mu - s1 + p - ff;
         if (gv > 0.0) a = mu;
         else if (gv < 0.0) b = mu;
         else break;
-        const double nw = mu - F / Fp;
-        if (fabs(nw - mu) <= 4.0 * kEpsD * fabs(mu)) {      // Newton step of a few ulps: converged
+        double A, B, C;
+        if (f >= 0) {
+            const double q = dl * (1.0 + s2) + ff;        // D delta, D = 1 + S2 + zeta_f / delta^2
+            A = p - q - gv;
+            B = gv * (dl - mu) - p * dl - q * mu;
+            C = gv * mu * dl;
+        } else {
+            A = -(1.0 + s2);
+            B = gv + A * mu - p;
+            C = gv * mu;
+        }
+        const double sq = sqrt(fmax(B * B - 4.0 * A * C, 0.0));
+        const double eta = -2.0 * C / (B + copysign(sq, B));
+        const double nw = mu + eta;
+        if (fabs(eta) <= 4.0 * kEpsD * fabs(mu)) {          // a step of a few ulps: converged
             if (nw >= a && nw <= b) mu = nw;
             break;
         }
-        const double nxt = (nw > a && nw < b) ? nw : 0.5 * (a + b);   // else bisection
-        mu = nxt;
+        if (nw > a && nw < b) {
+            mu = nw;
+        } else {                                            // else bisection: of the magnitudes, once the bracket
+            double mid = 0.5 * (a + b);                     // does not touch the pole (roots lie close to poles)
+            if (a * b > 0.0) {
+                const double gm = copysign(sqrt(a * b), a);
+                if (gm > a && gm < b) mid = gm;
+            }
+            mu = mid;
+        }
         if ((b - a) <= 4.0 * kEpsD * fmax(fabs(a), fabs(b))) break;
     }
     if (lane == 0) {
@@ -728,7 +817,7 @@ void outer_arrow_eig(const double* H, int ldh, int k, int w, double* theta, doub
     const int bytes = (int)(sizeof(double) * 2 * kMMax * kArrowLd);
     static std::once_flag once;
     std::call_once(once, [bytes] { cudaFuncSetAttribute(k_arrow_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
-    k_arrow_setup<<<w, kArrowThreads, bytes, s>>>(H, ldh, k, w, S, lds, aw, hs, off_cap);
+    k_arrow_setup<<<w, kArrowSetup, bytes, s>>>(H, ldh, k, w, S, lds, aw, hs, off_cap);
     int nl = 1;
     if (w < k) {
         k_arrow_roots<<<w + 1, 32, 0, s>>>(aw);

@@ -555,7 +555,7 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
             const bool one = slices_only(a.rs);          // gather and rows in one kernel
             if (one) ml_phase1_all<T>(a, h->lanes, s); else inner_gather<T>(a, h->lanes, s);
             if (prof) ck(cudaEventRecord(h->ev[4 * i + 1], s));
-            if (!one) ml_phase1<T>(a, s);
+            if (!one) ml_phase1<T>(a, s);                // else: the time counts as the gather's
             if (prof) ck(cudaEventRecord(h->ev[4 * i + 2], s));
             ml_second_phase<T>(h, b, a, 0, cudaGraphConditionalHandle{}, 0, s);
             if (prof) ck(cudaEventRecord(h->ev[4 * i + 3], s));
@@ -572,7 +572,7 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
                 ck(cudaEventElapsedTime(&ms_rows, h->ev[4 * i + 1], h->ev[4 * i + 2]));
                 ck(cudaEventElapsedTime(&ms_p2, h->ev[4 * i + 2], h->ev[4 * i + 3]));
                 h->stats.inner_phase1_ms += ms;
-                h->stats.inner_rows_ms += ms_rows;
+                if (!slices_only(a.rs)) h->stats.inner_rows_ms += ms_rows;
                 h->stats.inner_phase2_ms += ms_p2;
                 h->stats.inner_phase1_timed += 1;
                 h->stats.inner_phase1_csum += c;
@@ -905,6 +905,55 @@ void precond_apply_t(isira_handle h, InnerBuffers<T>& b, const T* d_x, T* d_y) {
         else ck(cudaMemcpyAsync(d_y, a.wv, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
     }
     sync(h);
+}
+}  // namespace
+
+namespace {
+// Scratch of isira_sym_eig_warm (36 KB), which has no handle to keep it: a call takes a free buffer of its
+// device and gives it back once its stream has been synchronised, so calls from any threads and streams
+// hold different buffers.  At most kArrowKept buffers are kept between calls; allocating and freeing
+// one on each call took longer than the Rayleigh-Ritz step.
+constexpr size_t kArrowKept = 16;
+struct ArrowPool {
+    std::mutex mu;
+    std::vector<std::pair<int, ArrowWork*>> kept;      // (device, buffer), arrival counter zero
+    ArrowPool() { kept.reserve(kArrowKept); }
+};
+ArrowPool& arrow_pool() {
+    static ArrowPool* p = new ArrowPool;                // outlives every thread that may still use it
+    return *p;
+}
+
+ArrowWork* take_arrow_work(int dev) {
+    {
+        ArrowPool& p = arrow_pool();
+        std::lock_guard<std::mutex> lk(p.mu);
+        for (size_t i = 0; i < p.kept.size(); ++i)
+            if (p.kept[i].first == dev) {
+                ArrowWork* aw = p.kept[i].second;
+                p.kept.erase(p.kept.begin() + (std::ptrdiff_t)i);
+                return aw;
+            }
+    }
+    ArrowWork* aw = nullptr;
+    if (cudaMalloc(&aw, sizeof(ArrowWork)) != cudaSuccess) return nullptr;
+    if (cudaMemset(aw, 0, sizeof(ArrowWork)) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) {
+        cudaFree(aw);
+        return nullptr;
+    }
+    return aw;
+}
+
+void give_arrow_work(int dev, ArrowWork* aw, bool clean) {
+    if (clean) {
+        ArrowPool& p = arrow_pool();
+        std::lock_guard<std::mutex> lk(p.mu);
+        if (p.kept.size() < kArrowKept) {
+            p.kept.push_back({dev, aw});
+            return;
+        }
+    }
+    cudaFree(aw);
 }
 }  // namespace
 
@@ -1570,15 +1619,13 @@ isira_status isira_sym_eig_warm(int k, int warm_w, const double* d_H, double* d_
     if (k < 2 || k > kMMax || warm_w < k - 1 || warm_w > k || !d_H || !d_theta || !d_S)
         return ISIRA_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    ArrowWork* aw = nullptr;
-    cudaError_t e = cudaMalloc(&aw, sizeof(ArrowWork));
-    if (e != cudaSuccess) return ISIRA_ERR_OOM;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return ISIRA_ERR_CUDA;
+    ArrowWork* aw = take_arrow_work(dev);
+    if (!aw) return ISIRA_ERR_OOM;
     int st = 1;
-    e = cudaMemsetAsync(aw, 0, sizeof(ArrowWork), s);
-    if (e == cudaSuccess) {
-        outer_arrow_eig(d_H, k, k, warm_w, d_theta, d_S, k, aw, nullptr, HUGE_VAL, nullptr, s);
-        e = cudaGetLastError();
-    }
+    outer_arrow_eig(d_H, k, k, warm_w, d_theta, d_S, k, aw, nullptr, HUGE_VAL, nullptr, s);
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&st, &aw->status, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess && st != 0) {
@@ -1586,7 +1633,7 @@ isira_status isira_sym_eig_warm(int k, int warm_w, const double* d_H, double* d_
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     }
-    cudaFree(aw);
+    give_arrow_work(dev, aw, e == cudaSuccess);
     if (path) *path = st == 0 ? 1 : 0;
     return e == cudaSuccess ? ISIRA_OK : ISIRA_ERR_CUDA;
 }
