@@ -158,9 +158,9 @@ def _ptr(t) -> int | None:
 # Every tensor handed to the library is checked here first (dtype, shape, layout, then device):
 # the C entry points take raw pointers and cannot tell a float32 buffer from a float64 one.
 
-def _check_tensor(t, name: str, dtypes: tuple, shape: tuple, cuda: bool = True):
+def _check_tensor(t, name: str, dtypes: tuple, shape: tuple, cuda: bool = True, contiguous: bool = True):
     """Raises ValueError unless t has one of `dtypes`, exactly `shape` (None = any extent in that
-    dimension), is contiguous and (with cuda) lives on a CUDA device."""
+    dimension), is contiguous (if asked for) and (with cuda) lives on a CUDA device."""
     import torch
     if not isinstance(t, torch.Tensor):
         raise ValueError(f"{name} must be a torch.Tensor")
@@ -169,7 +169,7 @@ def _check_tensor(t, name: str, dtypes: tuple, shape: tuple, cuda: bool = True):
     if t.dim() != len(shape) or any(want is not None and got != want for got, want in zip(t.shape, shape)):
         raise ValueError(f"{name} must have shape {tuple('*' if w is None else w for w in shape)}, "
                          f"not {tuple(t.shape)}")
-    if not t.is_contiguous():
+    if contiguous and not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
     if cuda:
         _check_cuda(**{name: t})
@@ -214,8 +214,8 @@ def _check_V(V, n: int, cmax: int = 31, cuda: bool = True):
     import torch
     if V is None:
         return 0
-    _check_tensor(V.contiguous() if isinstance(V, torch.Tensor) else V, "V", (torch.float64,), (n, None),
-                  cuda=cuda)
+    # any strides: the calls take V.t().contiguous(), a copy only where the columns are not contiguous already
+    _check_tensor(V, "V", (torch.float64,), (n, None), cuda=cuda, contiguous=False)
     if V.shape[1] > cmax:
         raise ValueError(f"V may have at most {cmax} columns, not {V.shape[1]}")
     return int(V.shape[1])
