@@ -682,19 +682,25 @@ __device__ __forceinline__ T pass_sum(const T (&v)[8], int r) {
     }
 }
 
-// the same with edge weights, products and sums in one operation
+// a product that the compiler may not fold into a following addition
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// the same with edge weights, products and sums in one operation where two entries pair up (a row's value
+// must not depend on how far its slice is padded: a zero entry adds nothing in either function, and a last
+// odd product is rounded as it would be beside one)
 template <typename T>
 __device__ __forceinline__ T pass_dot(const T (&v)[8], const T (&w)[8], int r) {
     auto two = [&](int u) { return fma(v[u + 1], w[u + 1], v[u] * w[u]); };
     switch (r) {
         case 0: return T(0);
-        case 1: return v[0] * w[0];
+        case 1: return mul_rn(v[0], w[0]);
         case 2: return two(0);
-        case 3: return fma(v[2], w[2], two(0));
+        case 3: return two(0) + mul_rn(v[2], w[2]);
         case 4: return two(0) + two(2);
-        case 5: return fma(v[4], w[4], two(0) + two(2));
+        case 5: return (two(0) + two(2)) + mul_rn(v[4], w[4]);
         case 6: return (two(0) + two(2)) + two(4);
-        case 7: return (two(0) + two(2)) + fma(v[6], w[6], two(4));
+        case 7: return (two(0) + two(2)) + (two(4) + mul_rn(v[6], w[6]));
         default: return (two(0) + two(2)) + (two(4) + two(6));
     }
 }

@@ -47,9 +47,13 @@ struct MlHierarchy {
 template <typename T>
 using GatherFn = std::function<void(const T* x, const T* res, T* g, cudaStream_t s)>;
 
+// visit (may be empty): the degree-descending number of every row, the order in which the aggregation goes
+// over the rows.  place (may be null): receives a numbering (new -> old) that keeps clusters together, where
+// the gathers of level 0 gain from it; the hierarchy is then built for that numbering (else it stays empty).
 template <typename T>
 cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci, const double* d_w, int64_t n,
-                     int64_t ld, int64_t skip, cudaStream_t s);
+                     int64_t ld, int64_t skip, const std::vector<int32_t>& visit, std::vector<int32_t>* place,
+                     cudaStream_t s);
 template <typename T> void ml_free(MlHierarchy<T>& H);
 // out = M^{-1} b, one V-cycle; kernels return at once while *done != 0 (done may be null)
 template <typename T>
@@ -181,6 +185,7 @@ struct OuterArgs {
     RowSched rs;
     double* gsum;               // per-row neighbour sums of the gather kernel
     int64_t n, ld;              // leading dimension of U, W, V
+    const int32_t* visit;       // row -> its number in the degree-descending order (null: the same)
     double* U; double* W; double* V;
     double* H;                  // kMMax x kMMax, column-major, ld kMMax
     double* theta; double* S;   // Ritz values, Ritz vectors (ld kMMax)
@@ -266,6 +271,10 @@ void setup_partition(const int64_t* rp, int64_t n, const int32_t* item_row, cons
 cudaError_t build_reordered_graph(const int64_t* rp, const int32_t* ci, const double* w, int64_t n, int64_t nnz,
                                   int64_t maxdeg, int64_t* rp2, int32_t* ci2, double* w2, int32_t* perm, int32_t* inv,
                                   cudaStream_t s);
+// the relabelled graph relabelled again by order (new -> old of its numbering; rows keep their entries' order)
+cudaError_t build_permuted_graph(const int64_t* rp, const int32_t* ci, const double* w, int64_t n, const int32_t* perm,
+                                 const int32_t* order, int64_t* rp2, int32_t* ci2, double* w2, int32_t* perm2,
+                                 int32_t* inv2, cudaStream_t s);
 // sliced ELL copy of the light rows [light0, n): off (n_slices + 1 entries, caller-allocated) receives
 // the slice offsets, *sci a new device array of *total entries (-1 padding)
 cudaError_t build_sell(const int64_t* rp, const int32_t* ci, const double* w, int64_t n, int64_t light0,

@@ -465,9 +465,70 @@ static void upload_i(I** dst, const std::vector<I>& src) {
     if (!src.empty()) CUDA_OK(cudaMemcpy(*dst, src.data(), sizeof(I) * src.size(), cudaMemcpyHostToDevice));
 }
 
+// Sampled cost of level 0's gathers in a numbering (order: new -> old; null: as it is): the 128-byte lines that
+// the warp-wide loads of x touch, counting a column of a slice, also a padded one, as at least one; *cols
+// receives the number of columns.
+static int64_t gather_lines(const HostLevel& A, const std::vector<int32_t>* order, const std::vector<int32_t>& pos,
+                            int64_t* cols) {
+    const int64_t ns = A.n / 32, step = std::max<int64_t>(1, ns / 256);
+    int64_t lines = 0;
+    int32_t ln[32];
+    *cols = 0;
+    for (int64_t s = 0; s < ns; s += step) {
+        int64_t wid = 0;
+        for (int64_t r = 32 * s; r < 32 * s + 32; ++r) {
+            const int64_t i = order ? (*order)[r] : r;
+            wid = std::max(wid, A.rp[i + 1] - A.rp[i]);
+        }
+        *cols += wid;
+        for (int64_t q = 0; q < wid; ++q) {
+            int m = 0;
+            for (int64_t r = 32 * s; r < 32 * s + 32; ++r) {
+                const int64_t i = order ? (*order)[r] : r;
+                if (A.rp[i] + q < A.rp[i + 1]) {
+                    const int32_t c = A.ci[A.rp[i] + q];
+                    ln[m++] = (order ? pos[c] : c) >> 5;
+                }
+            }
+            std::sort(ln, ln + m);
+            lines += std::max<int64_t>(1, std::unique(ln, ln + m) - ln);
+        }
+    }
+    return lines;
+}
+
+// A numbering of level 0 that keeps clusters, and clusters of clusters, together (level 1's numbers are
+// hierarchical), with the rows of every kMlWindow consecutive ones by descending degree, so that the slices of
+// 32 rows stay nearly unpadded.
+constexpr int64_t kMlWindow = 128;
+
+static std::vector<int32_t> cluster_order(const HostLevel& A, const std::vector<int32_t>& agg, int64_t nc) {
+    std::vector<int64_t> start(nc + 2, 0);                 // the excluded vertex (-1) goes last
+    for (int64_t i = 0; i < A.n; ++i) start[(agg[i] < 0 ? nc : agg[i]) + 1]++;
+    for (int64_t I = 0; I <= nc; ++I) start[I + 1] += start[I];
+    std::vector<int32_t> order(A.n);
+    for (int64_t i = 0; i < A.n; ++i) order[start[agg[i] < 0 ? nc : agg[i]]++] = (int32_t)i;
+    // counting sort of each window (all rows are sliced: degrees up to 64)
+    constexpr int kDeg = 65;
+    int32_t deg[kMlWindow], row[kMlWindow];
+    for (int64_t w = 0; w < A.n; w += kMlWindow) {
+        const int m = (int)std::min(kMlWindow, A.n - w);
+        int cnt[kDeg + 1] = {};
+        for (int t = 0; t < m; ++t) {
+            row[t] = order[w + t];
+            deg[t] = kDeg - 1 - (int32_t)std::min<int64_t>(kDeg - 1, A.rp[row[t] + 1] - A.rp[row[t]]);
+            ++cnt[deg[t] + 1];
+        }
+        for (int d = 0; d < kDeg; ++d) cnt[d + 1] += cnt[d];
+        for (int t = 0; t < m; ++t) order[w + cnt[deg[t]]++] = row[t];
+    }
+    return order;
+}
+
 template <typename T>
 cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci, const double* d_w, int64_t n,
-                     int64_t ld, int64_t skip, cudaStream_t s) {
+                     int64_t ld, int64_t skip, const std::vector<int32_t>& visit, std::vector<int32_t>* place,
+                     cudaStream_t s) {
     try {
         HostLevel A0;
         A0.n = n;
@@ -482,17 +543,37 @@ cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci
             CUDA_OK(cudaMemcpyAsync(A0.w.data(), d_w, sizeof(double) * A0.rp[n], cudaMemcpyDeviceToHost, s));
             CUDA_OK(cudaStreamSynchronize(s));
         }
+        // the rows in their degree-descending order (old); pos: old -> the numbering in use
+        std::vector<int32_t> order = visit, pos;
+        if (!order.empty()) {
+            pos.resize(n);
+            for (int64_t r = 0; r < n; ++r) pos[order[r]] = (int32_t)r;
+            HostLevel B;
+            B.n = n;
+            B.rp.assign(n + 1, 0);
+            B.ci.resize(A0.ci.size());
+            B.w.resize(A0.w.size());
+            for (int64_t i = 0; i < n; ++i) {
+                int64_t e2 = B.rp[i];
+                for (int64_t e = A0.rp[pos[i]]; e < A0.rp[pos[i] + 1]; ++e, ++e2) {
+                    B.ci[e2] = order[A0.ci[e]];
+                    B.w[e2] = A0.w[e];
+                }
+                B.rp[i + 1] = e2;
+            }
+            A0 = std::move(B);
+        }
+        const int64_t skip_old = order.empty() || skip < 0 ? skip : order[skip];
         A0.d.assign(n, 0.0);
         for (int64_t i = 0; i < n; ++i)
             for (int64_t e = A0.rp[i]; e < A0.rp[i + 1]; ++e) A0.d[i] += A0.w[e];
         H.n0 = n;
-        H.skip = skip;
         std::vector<HostLevel> levels;
         levels.push_back(std::move(A0));
         std::vector<std::vector<int32_t>> aggs;
         while ((int)levels.size() < kMlMaxLevels && levels.back().n > kMlCoarse) {
             int64_t nc = 0;
-            const int64_t sk = levels.size() == 1 ? skip : -1;
+            const int64_t sk = levels.size() == 1 ? skip_old : -1;
             std::vector<int32_t> agg = aggregate(levels.back(), sk, &nc);
             if (nc >= levels.back().n * 9 / 10 || nc < 1) break;    // no useful coarsening left
             HostLevel C = coarsen(levels.back(), agg, nc);
@@ -533,6 +614,25 @@ cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci
                 if (x >= 0) x = (int32_t)pos[x];
         }
         const int L = (int)levels.size();
+        if (place) {
+            place->clear();
+            // Worth the second relabelling where it halves the lines.  A random geometric graph numbered at random
+            // touches a line per entry (45 us a gather of 1M vertices, 41 us of them lines at one per cycle and
+            // SM; 20 us relabelled); a grid in its own order touches two or three per column of a slice, which
+            // no numbering halves: below six the order is not even formed.
+            int64_t cols = 0, cols_new = 0;
+            const int64_t lines = L > 1 && order.empty() ? gather_lines(levels[0], nullptr, pos, &cols) : 0;
+            if (lines >= 6 * std::max<int64_t>(1, cols)) {
+                std::vector<int32_t> o = cluster_order(levels[0], aggs[0], levels[1].n), p(n);
+                for (int64_t r = 0; r < n; ++r) p[o[r]] = (int32_t)r;
+                if (2 * gather_lines(levels[0], &o, p, &cols_new) < lines) {
+                    *place = o;
+                    order = std::move(o);
+                    pos = std::move(p);
+                }
+            }
+        }
+        H.skip = order.empty() || skip_old < 0 ? skip_old : pos[skip_old];
         H.nlev = L;
         H.lev.assign(L, MlLevel<T>{});
         for (int l = 0; l < L; ++l) {
@@ -541,7 +641,8 @@ cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci
             D.n = A.n;
             D.nnz = (int64_t)A.ci.size();
             std::vector<double> dinv(l == 0 ? ld : A.n, 0.0);
-            for (int64_t i = 0; i < A.n; ++i) dinv[i] = (l == 0 && i == skip) ? 0.0 : 1.0 / A.d[i];
+            auto place_of = [&](int64_t i) { return l == 0 && !pos.empty() ? (int64_t)pos[i] : i; };
+            for (int64_t i = 0; i < A.n; ++i) dinv[place_of(i)] = (l == 0 && i == skip_old) ? 0.0 : 1.0 / A.d[i];
             upload<T>(&D.dinv, dinv);
             if (l > 0) {
                 std::vector<int32_t> rp32(A.n + 1);
@@ -560,7 +661,7 @@ cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci
             if (l + 1 < L) {
                 const std::vector<int32_t>& agg = aggs[l];
                 std::vector<int32_t> agg_pad(nv, -1);
-                std::copy(agg.begin(), agg.end(), agg_pad.begin());
+                for (int64_t i = 0; i < (int64_t)agg.size(); ++i) agg_pad[place_of(i)] = agg[i];
                 upload_i<int32_t>(&D.agg, agg_pad);
                 const int64_t nc = levels[l + 1].n;
                 std::vector<int64_t> mrp(nc + 1, 0);
@@ -568,15 +669,15 @@ cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci
                     if (I >= 0) mrp[I + 1]++;
                 for (int64_t I = 0; I < nc; ++I) mrp[I + 1] += mrp[I];
                 std::vector<int32_t> mem(mrp[nc]);
-                std::vector<int64_t> pos(mrp.begin(), mrp.end() - 1);
+                std::vector<int64_t> fill(mrp.begin(), mrp.end() - 1);
                 for (int64_t i = 0; i < (int64_t)agg.size(); ++i)
-                    if (agg[i] >= 0) mem[pos[agg[i]]++] = (int32_t)i;
+                    if (agg[i] >= 0) mem[fill[agg[i]]++] = (int32_t)place_of(i);   // members in the old order
                 upload_i<int64_t>(&D.mrp, mrp);
                 upload_i<int32_t>(&D.mem, mem);
             }
         }
         std::vector<double> inv;
-        if (!dense_inverse(levels[L - 1], L == 1 ? skip : -1, inv)) return cudaErrorInvalidValue;
+        if (!dense_inverse(levels[L - 1], L == 1 ? skip_old : -1, inv)) return cudaErrorInvalidValue;
         upload<T>(&H.inv, inv);
         H.n_coarse = levels[L - 1].n;
         CUDA_OK(cudaStreamSynchronize(s));
@@ -687,7 +788,8 @@ void ml_stage(MlHierarchy<T>& H, const T* x, const int32_t* perm, T omega, T* b,
 
 #define ISIRA_INSTANTIATE_ML(T)                                                                              \
     template cudaError_t ml_build<T>(MlHierarchy<T>&, const int64_t*, const int32_t*, const double*, int64_t,  \
-                                     int64_t, int64_t, cudaStream_t);                                        \
+                                     int64_t, int64_t, const std::vector<int32_t>&, std::vector<int32_t>*,   \
+                                     cudaStream_t);                                                          \
     template void ml_free<T>(MlHierarchy<T>&);                                                               \
     template void ml_vcycle<T>(MlHierarchy<T>&, const T*, T*, const GatherFn<T>&, T, T, const int*, bool,     \
                                bool, const int32_t*, cudaStream_t);                                          \

@@ -1288,13 +1288,14 @@ void outer_set_diag(const OuterArgs& a, int c0, int cnt, cudaStream_t s) {
     k_set_diag<<<1, kThreads, 0, s>>>(a.H, a.theta, a.S, c0, cnt);
 }
 
-__global__ void k_random(double* Z, int64_t n, uint64_t seed, uint64_t blk) {
+// entry r comes from the counter of the row's degree-descending number, whatever numbering is in use
+__global__ void k_random(double* Z, const int32_t* __restrict__ visit, int64_t n, uint64_t seed, uint64_t blk) {
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-        Z[r] = 2.0 * uniform_at(seed, blk * (uint64_t)n + (uint64_t)r) - 1.0;
+        Z[r] = 2.0 * uniform_at(seed, blk * (uint64_t)n + (uint64_t)(visit ? visit[r] : r)) - 1.0;
 }
 
 void outer_random(const OuterArgs& a, uint64_t seed, uint64_t blk, cudaStream_t s) {
-    k_random<<<a.ew_blocks, kThreads, 0, s>>>(a.Z, a.n, seed, blk);
+    k_random<<<a.ew_blocks, kThreads, 0, s>>>(a.Z, a.visit, a.n, seed, blk);
 }
 
 // ------------------------------------------------------------------ true residual

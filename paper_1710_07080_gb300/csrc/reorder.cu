@@ -57,6 +57,43 @@ __global__ void k_scatter_perm(const T* src, const int32_t* perm, int64_t n, T* 
         dst[perm[i]] = src[i];
 }
 
+// perm2[i] = perm[order[i]] and its inverse: the caller's number of the row that a second relabelling put at i
+__global__ void k_compose_perm(const int32_t* perm, const int32_t* order, int64_t n, int32_t* perm2, int32_t* inv2) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t u = perm[order[i]];
+        perm2[i] = u;
+        inv2[u] = (int32_t)i;
+    }
+}
+
+cudaError_t build_permuted_graph(const int64_t* rp, const int32_t* ci, const double* w, int64_t n, const int32_t* perm,
+                                 const int32_t* order, int64_t* rp2, int32_t* ci2, double* w2, int32_t* perm2,
+                                 int32_t* inv2, cudaStream_t s) {
+    int64_t* deg = nullptr;
+    int32_t* pos = nullptr;
+    void* tmp = nullptr;
+    size_t bytes = 0;
+    cudaError_t e = cudaSuccess;
+    const int grid = 1024;
+#define CK(x) do { e = (x); if (e != cudaSuccess) goto done; } while (0)
+    CK(cudaMalloc(&deg, sizeof(int64_t) * (size_t)(n + 1)));
+    CK(cudaMalloc(&pos, sizeof(int32_t) * (size_t)n));
+    CK(cub::DeviceScan::ExclusiveSum(nullptr, bytes, deg, rp2, (int)(n + 1), s));
+    CK(cudaMalloc(&tmp, bytes));
+    k_new_degrees<<<grid, kThreads, 0, s>>>(rp, order, n, deg, pos);
+    CK(cub::DeviceScan::ExclusiveSum(tmp, bytes, deg, rp2, (int)(n + 1), s));
+    k_permute_cols<<<grid, kThreads, 0, s>>>(rp, ci, w, order, pos, rp2, n, ci2, w2);
+    k_compose_perm<<<grid, kThreads, 0, s>>>(perm, order, n, perm2, inv2);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(s));
+#undef CK
+done:
+    if (deg) cudaFree(deg);
+    if (pos) cudaFree(pos);
+    if (tmp) cudaFree(tmp);
+    return e;
+}
+
 cudaError_t build_reordered_graph(const int64_t* rp, const int32_t* ci, const double* w, int64_t n, int64_t nnz,
                                   int64_t maxdeg, int64_t* rp2, int32_t* ci2, double* w2, int32_t* perm, int32_t* inv,
                                   cudaStream_t s) {

@@ -93,6 +93,9 @@ struct isira_handle_s {
     int32_t* own_ci = nullptr;
     int32_t* perm = nullptr;
     int32_t* inv = nullptr;
+    // second relabelling by clusters (relocate): row -> its degree-descending number, host and device
+    std::vector<int32_t> visit;
+    int32_t* visit_dev = nullptr;
     int64_t trim_user = 0;
     int64_t n_long = 0, n_items = 0;
     RowSched rs{};
@@ -218,6 +221,7 @@ OuterArgs make_outer(isira_handle h) {
     a.rs = h->rs;
     a.n = h->n;
     a.ld = h->ld;
+    a.visit = h->visit_dev;
     a.U = h->U; a.W = h->W; a.V = h->V;
     a.H = h->H; a.theta = h->theta; a.S = h->S;
     a.R = h->R; a.Z = h->Z;
@@ -433,15 +437,91 @@ int run_inner(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* 
 
 // ------------------------------------------------------------------ multilevel-preconditioned inner solve
 
+// Takes the solver's copy of the graph (all rows sliced) into the numbering `place` (new -> old of the
+// present one).  Called in create before anything but the hierarchy depends on the numbering: rows keep their
+// entries' order and the clusters their members', so operator and V-cycle give the same sums as before.
+void relocate(isira_handle h, std::vector<int32_t> place) {
+    cudaStream_t s = h->stream;
+    const int64_t n = h->n;
+    int32_t *order = nullptr, *perm2 = nullptr, *inv2 = nullptr;
+    int64_t* rp2 = nullptr;
+    int32_t* ci2 = nullptr;
+    double* w2 = nullptr;
+    const size_t nnz_pad = ((size_t)h->nnz + 3) / 4 * 4;
+    auto drop = [&] {
+        void* p[] = {order, perm2, inv2, rp2, ci2, w2};
+        for (void* q : p)
+            if (q) cudaFree(q);
+    };
+    try {
+        ck(cudaMalloc(&order, sizeof(int32_t) * (size_t)n));
+        ck(cudaMalloc(&perm2, sizeof(int32_t) * (size_t)n));
+        ck(cudaMalloc(&inv2, sizeof(int32_t) * (size_t)n));
+        ck(cudaMalloc(&rp2, sizeof(int64_t) * (size_t)(n + 1)));
+        ck(cudaMalloc(&ci2, sizeof(int32_t) * nnz_pad));
+        if (h->own_w) ck(cudaMalloc(&w2, sizeof(double) * (size_t)h->nnz));
+        ck(cudaMemcpyAsync(order, place.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, s));
+        ck(cudaMemsetAsync(ci2 + h->nnz, 0, sizeof(int32_t) * (nnz_pad - (size_t)h->nnz), s));
+        ck(build_permuted_graph(h->own_rp, h->own_ci, h->own_w, n, h->perm, order, rp2, ci2, w2, perm2, inv2, s));
+    } catch (...) {
+        drop();
+        throw;
+    }
+    std::swap(h->own_rp, rp2);
+    std::swap(h->own_ci, ci2);
+    std::swap(h->own_w, w2);
+    std::swap(h->perm, perm2);
+    std::swap(h->inv, inv2);
+    std::swap(h->visit_dev, order);
+    drop();                                               // the old arrays
+    int64_t t = 0;
+    while (place[(size_t)t] != h->trim) ++t;
+    h->trim = t;
+    h->visit = std::move(place);
+    RowSched& rs = h->rs;
+    rs.rp = h->rp = h->own_rp;
+    rs.ci = h->ci = h->own_ci;
+    setup_deg32(h->own_rp, n, h->ld, h->deg32, s);
+    if (h->own_w) {
+        rs.wd = h->own_w;
+        setup_weighted(h->own_rp, h->own_w, n, h->ld, h->nnz, h->degwd, h->degwf, h->wf, s);
+    }
+    void* sell[] = {h->sell_ci, h->sell_wd, h->sell_wf};
+    for (void* p : sell)
+        if (p) cudaFree(p);
+    h->sell_ci = nullptr;
+    h->sell_wd = nullptr;
+    h->sell_wf = nullptr;
+    ck(build_sell(h->own_rp, h->own_ci, h->own_w, n, 0, rs.n_slices, h->sell_off, &h->sell_ci,
+                  h->own_w ? &h->sell_wd : nullptr, &h->sell_total, s));
+    if (h->own_w) {
+        ck(cudaMalloc(&h->sell_wf, sizeof(float) * (size_t)std::max<int64_t>(1, h->sell_total)));
+        copy_cast<float>(h->sell_wd, h->sell_wf, h->sell_total, s);
+        rs.swd = h->sell_wd;
+        rs.swf = h->sell_wf;
+    }
+    rs.sell_ci = h->sell_ci;
+    unsigned long long* scr = reinterpret_cast<unsigned long long*>(h->dscratch);
+    cluster_plan<float>(rs, h->sell_total, scr, s, &h->cl_f);
+    cluster_plan<double>(rs, h->sell_total, scr, s, &h->cl_d);
+}
+
+// may_place: in create, while the numbering may still change
 template <typename T>
-void ensure_ml(isira_handle h, InnerBuffers<T>& b) {
+void ensure_ml(isira_handle h, InnerBuffers<T>& b, bool may_place = false) {
     if (!b.ml) {
         const size_t elems = (size_t)h->ld * 4;
         ck(cudaMalloc(&b.ml, sizeof(T) * elems));
         ck(cudaMemsetAsync(b.ml, 0, sizeof(T) * elems, h->stream));
     }
     if (!h->ml_dv) ck(cudaMalloc(&h->ml_dv, sizeof(double) * kCMax));
-    if (b.H.nlev == 0) ck(ml_build<T>(b.H, h->rs.rp, h->rs.ci, h->rs.wd, h->n, h->ld, h->trim, h->stream));
+    if (b.H.nlev == 0) {
+        std::vector<int32_t> place;
+        may_place = may_place && h->perm && slices_only(h->rs) && h->visit.empty();
+        ck(ml_build<T>(b.H, h->rs.rp, h->rs.ci, h->rs.wd, h->n, h->ld, h->trim, h->visit, may_place ? &place : nullptr,
+                       h->stream));
+        if (!place.empty()) relocate(h, std::move(place));
+    }
 }
 
 template <typename T>
@@ -613,7 +693,7 @@ void choose_preconditioner(isira_handle h) {
     const int pc = h->opts.precond;
     const bool mixed = h->opts.precision == ISIRA_MIXED;
     auto build = [&]() {
-        if (mixed) ensure_ml(h, h->fb); else ensure_ml(h, h->db);
+        if (mixed) ensure_ml(h, h->fb, true); else ensure_ml(h, h->db, true);
         sync(h);
     };
     h->use_ml = false;
@@ -814,7 +894,7 @@ void autotune_gather(isira_handle h) {
 
 void free_handle(isira_handle h) {
     if (!h) return;
-    void* ptrs[] = {h->vbuf, h->own_w, h->wf, h->degwd, h->degwf, h->sell_wd, h->sell_wf, h->gsum, h->deg32, h->sell_off, h->sell_ci, h->own_rp, h->own_ci, h->perm, h->inv, h->item_row, h->item_k, h->item_partial,
+    void* ptrs[] = {h->visit_dev, h->vbuf, h->own_w, h->wf, h->degwd, h->degwf, h->sell_wd, h->sell_wf, h->gsum, h->deg32, h->sell_off, h->sell_ci, h->own_rp, h->own_ci, h->perm, h->inv, h->item_row, h->item_k, h->item_partial,
                     h->item_count, h->warp_start, h->U, h->W, h->V, h->H, h->theta, h->S, h->R, h->Z, h->dscratch,
                     h->arrow, h->partial, h->counter, h->Gm, h->Cinv, h->lam_dev, h->tres_dev, h->fb.base, h->fb.st,
                     h->db.base, h->db.st, h->Vt_f, h->fb.ml, h->db.ml, h->ml_dv};
