@@ -553,6 +553,7 @@ __global__ void __launch_bounds__(kThreads) k_sell_lines(const int32_t* __restri
 //  * FP64 up to 30,720 rows: 16 SMs issue the FP64 instructions of 152, so the line is where that costs what
 //    the launches did (grids of 9,856 / 30,600 vertices: 9.3 / 19.7 and 18.3 / 42.7 us against 27 / 40 and 29 / 44 us;
 //    ER of 40,000: 34 / 64 against 32 / 46 us).
+//    (The launches' times are those with one iteration a turn of the WHILE node; four take 2 to 3 us off.)
 //  * CTAs: enough for 256 rows each in FP32 (latency) and 64 in FP64 (its narrow pipe), 16 at most.
 //  * Staging copies z_k whole into every CTA's shared memory each iteration and gathers from there: it pays
 //    in FP32 when the gathers touch more lines than the copy moves (ER of 12,339: 4.7 us against 6.6 us; grid of

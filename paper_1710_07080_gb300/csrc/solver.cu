@@ -444,7 +444,8 @@ int run_inner(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* 
 // Takes the solver's copy of the graph (all rows sliced) into the numbering `place` (new -> old of the
 // present one).  Called in create before anything but the hierarchy depends on the numbering: rows keep their
 // entries' order and the clusters their members', so operator and V-cycle give the same sums as before.
-void relocate(isira_handle h, std::vector<int32_t> place) {
+// False, with nothing changed, if there is no memory for the second copy.
+bool relocate(isira_handle h, std::vector<int32_t> place) {
     cudaStream_t s = h->stream;
     const int64_t n = h->n;
     int32_t *order = nullptr, *perm2 = nullptr, *inv2 = nullptr;
@@ -467,9 +468,11 @@ void relocate(isira_handle h, std::vector<int32_t> place) {
         ck(cudaMemcpyAsync(order, place.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, s));
         ck(cudaMemsetAsync(ci2 + h->nnz, 0, sizeof(int32_t) * (nnz_pad - (size_t)h->nnz), s));
         ck(build_permuted_graph(h->own_rp, h->own_ci, h->own_w, n, h->perm, order, rp2, ci2, w2, perm2, inv2, s));
-    } catch (...) {
+    } catch (const CudaError& e) {
         drop();
-        throw;
+        if (e.e != cudaErrorMemoryAllocation) throw;
+        cudaGetLastError();
+        return false;
     }
     std::swap(h->own_rp, rp2);
     std::swap(h->own_ci, ci2);
@@ -508,6 +511,7 @@ void relocate(isira_handle h, std::vector<int32_t> place) {
     unsigned long long* scr = reinterpret_cast<unsigned long long*>(h->dscratch);
     cluster_plan<float>(rs, h->sell_total, scr, s, &h->cl_f);
     cluster_plan<double>(rs, h->sell_total, scr, s, &h->cl_d);
+    return true;
 }
 
 // may_place: in create, while the numbering may still change
@@ -524,7 +528,10 @@ void ensure_ml(isira_handle h, InnerBuffers<T>& b, bool may_place = false) {
         may_place = may_place && h->perm && slices_only(h->rs) && h->visit.empty();
         ck(ml_build<T>(b.H, h->rs.rp, h->rs.ci, h->rs.wd, h->n, h->ld, h->trim, h->visit, may_place ? &place : nullptr,
                        h->stream));
-        if (!place.empty()) relocate(h, std::move(place));
+        if (!place.empty() && !relocate(h, std::move(place))) {
+            ml_free<T>(b.H);
+            ck(ml_build<T>(b.H, h->rs.rp, h->rs.ci, h->rs.wd, h->n, h->ld, h->trim, h->visit, nullptr, h->stream));
+        }
     }
 }
 
