@@ -11,10 +11,11 @@
 // Scratch: the cross-CTA partial sums of 1^T x and Vh^T x live in the file-scope array
 // g_isira_noalloc_scratch below (about 72 KB).  Every GPU that loads this library holds that
 // array until the process exits.  Every call shares it, and it keeps the previous call's
-// contents: the arrival counter starts at zero and every launch leaves it there (no memset per call), and
-// every partial is written before it is read.  Calls whose work
+// contents: every partial is written before it is read, and the second kernel of every call, which is
+// ordered after the reduction, leaves the arrival counter at zero (no memset per call).  Calls whose work
 // overlaps on the GPU (two streams, two host threads) race on the array and give wrong
-// results; serialise them.
+// results; serialise them.  They leave no damage behind: whatever the counter holds after a race, the
+// second kernels of the racing calls clear it, so a later call that runs alone is right again.
 //
 // Device address: in host code the name g_isira_noalloc_scratch is only a host-side stand-in,
 // not a device address.  The first call on each device (with that device current) looks the
@@ -80,8 +81,9 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads) k_na_apply(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                        int64_t n, int64_t trim, T sigma, T sig_n, T delta,
                                                        const T* __restrict__ x, const double* __restrict__ V, int c,
-                                                       const double* scratch, T* __restrict__ y) {
+                                                       double* scratch, T* __restrict__ y) {
     constexpr int G = 4;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<unsigned*>(scratch + kNaCounter) = 0u;
     const T* coef = reinterpret_cast<const T*>(scratch + kNaCoef);
     const int lane = threadIdx.x & 31;
     const int64_t group = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
