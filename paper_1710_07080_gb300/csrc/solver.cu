@@ -733,12 +733,23 @@ void choose_preconditioner(isira_handle h) {
     h->stats.precond_probe_ms[1] = t[1];
 }
 
+// The inner graphs hold the address of the deflation vectors (V, Vt_f) in their kernels' arguments: once these
+// move, every graph but that of rank 0, which reads none, has to be captured again.
+void drop_inner_graphs(isira_handle h) {
+    for (cudaGraphExec_t* graphs : {h->inner_graph, h->ml_graph})
+        for (int b = 1; b < 6; ++b) {
+            if (graphs[b]) cudaGraphExecDestroy(graphs[b]);
+            graphs[b] = nullptr;
+        }
+}
+
 void ensure_outer(isira_handle h, int m, int d) {
     const size_t ld = (size_t)h->ld;
     if (m > h->m_alloc) {
         if (h->U) cudaFree(h->U);
         if (h->W) cudaFree(h->W);
         h->U = h->W = nullptr;
+        h->m_alloc = 0;
         ck(cudaMalloc(&h->U, sizeof(double) * ld * m));
         ck(cudaMalloc(&h->W, sizeof(double) * ld * m));
         h->m_alloc = m;
@@ -748,6 +759,8 @@ void ensure_outer(isira_handle h, int m, int d) {
         if (h->Vt_f) cudaFree(h->Vt_f);
         h->V = nullptr;
         h->Vt_f = nullptr;
+        h->d_alloc = 0;
+        drop_inner_graphs(h);
         ck(cudaMalloc(&h->V, sizeof(double) * ld * d));
         if (h->opts.precision == ISIRA_MIXED) ck(cudaMalloc(&h->Vt_f, sizeof(float) * ld * d));
         h->d_alloc = d;
