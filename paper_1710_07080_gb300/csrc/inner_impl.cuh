@@ -664,11 +664,18 @@ constexpr int kGramBlocks = 456;        // three CTAs per SM: the last CTA adds 
 // shared memory; the c (c + 1) / 2 entries are dealt to the threads, several row segments to an entry
 // while there are threads left (c = 4: 25 segments of 10 entries; one thread per entry, as before, left 246 of 256
 // idle and the Cholesky factorisation and the inverse to a single one).  The last CTA factors C with
-// one lane per row and inverts it with one lane per column.  Bound by the FP64 pipe: n c^2 / 2 FMAs.
+// one lane per row and inverts it with one lane per column, in the tile's place (at most 2 c (c + 2)
+// of its 129 c doubles).  Bound by the FP64 pipe: n c^2 / 2 FMAs.  All of its shared memory fits the 48 KB that a launch
+// may take without a function attribute, which would hold for one device of the process only.
+constexpr int kGramLd = kGramTile + 1;
+constexpr size_t gram_smem(int c) { return sizeof(double) * (size_t)c * kGramLd; }
+static_assert(2 * (kCMax - 1) * (kCMax + 1) <= (kCMax - 1) * kGramLd, "C and its inverse's columns need the tile's room");
+static_assert(gram_smem(kCMax - 1) + sizeof(double) * (kGramTile + 2 * kThreads) + 64 <= 48 * 1024, "no opt-in");
+
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_gram(InnerArgs<T> a, double* G, double* Cinv, double* partial,
                                                    int pstride) {
-    extern __shared__ double gsm[];     // [c][kGramTile + 1]
+    extern __shared__ double gsm[];     // [c][kGramLd]
     __shared__ double rs[kGramTile];
     __shared__ double red[2 * kThreads];
     const int c = a.c, tid = threadIdx.x;
@@ -692,7 +699,7 @@ __global__ void __launch_bounds__(kThreads) k_gram(InnerArgs<T> a, double* G, do
             eb[q] = p + rem;
         }
     }
-    const int ldt = kGramTile + 1;
+    constexpr int ldt = kGramLd;
     for (int64_t r0 = (int64_t)blockIdx.x * kGramTile; r0 < n; r0 += (int64_t)gridDim.x * kGramTile) {
         __syncthreads();
         for (int rr = tid; rr < kGramTile; rr += kThreads) {
@@ -740,8 +747,9 @@ __global__ void __launch_bounds__(kThreads) k_gram(InnerArgs<T> a, double* G, do
     __syncthreads();
     if (!last) return;
     last_block_sum(partial, pstride, gridDim.x, ne, red, a.counter);
-    constexpr int L = kCMax + 1;
-    __shared__ double A[kCMax * L], Y[kCMax * L];
+    const int L = (c + 1) | 1;            // odd: lanes read columns without bank conflicts
+    double* A = gsm;
+    double* Y = gsm + c * L;
     const double dinv = 1.0 / (double)a.delta;
     for (int e = tid; e < ne; e += kThreads) {
         const double s = red[e];
@@ -1663,13 +1671,7 @@ void stage_inputs(const double* r_in, const double* V, const int32_t* perm, int6
 template <typename T>
 void gram_setup(const InnerArgs<T>& a, double* G_out, double* Cinv_out, double* partial, cudaStream_t s) {
     if (a.c <= 0) return;
-    const size_t smem = sizeof(double) * (size_t)a.c * (kGramTile + 1);
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_gram<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * kCMax * (kGramTile + 1)));
-    });
-    k_gram<T><<<std::min(a.ew_blocks, kGramBlocks), kThreads, smem, s>>>(a, G_out, Cinv_out, partial, a.pstride);
+    k_gram<T><<<std::min(a.ew_blocks, kGramBlocks), kThreads, gram_smem(a.c), s>>>(a, G_out, Cinv_out, partial, a.pstride);
 }
 
 template <typename T>
