@@ -11,8 +11,8 @@
 //   setup         degrees, maximum degree and its vertex, row classes (Remark 4.1)
 // The tall-skinny kernels give a thread whole rows and go over the columns in batches held in registers.
 #include <algorithm>
-#include <mutex>
 
+#include "device_once.h"
 #include "internal.h"
 
 namespace isira {
@@ -300,8 +300,8 @@ __global__ void __launch_bounds__(kEigThreads) k_sym_eig(const double* H, int ld
 void outer_sym_eig(const double* H, int ldh, int k, double* theta, double* S, int lds, HostStatus* hs,
                    int warm_w, cudaStream_t s) {
     const int bytes = (int)(sizeof(double) * 5 * kMMax * kEigLd);
-    static std::once_flag once;
-    std::call_once(once, [bytes] { cudaFuncSetAttribute(k_sym_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+    static PerDeviceOnce once;
+    once([bytes] { return cudaFuncSetAttribute(k_sym_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
     k_sym_eig<<<1, kEigThreads, bytes, s>>>(H, ldh, k, theta, S, lds, hs, warm_w);
 }
 
@@ -815,8 +815,8 @@ __global__ void __launch_bounds__(kArrowThreads) k_arrow_vectors(int k, int w, A
 void outer_arrow_eig(const double* H, int ldh, int k, int w, double* theta, double* S, int lds, ArrowWork* aw,
                      HostStatus* hs, double off_cap, int* launches, cudaStream_t s) {
     const int bytes = (int)(sizeof(double) * 2 * kMMax * kArrowLd);
-    static std::once_flag once;
-    std::call_once(once, [bytes] { cudaFuncSetAttribute(k_arrow_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+    static PerDeviceOnce once;
+    once([bytes] { return cudaFuncSetAttribute(k_arrow_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
     k_arrow_setup<<<w, kArrowSetup, bytes, s>>>(H, ldh, k, w, S, lds, aw, hs, off_cap);
     int nl = 1;
     if (w < k) {
@@ -1173,10 +1173,10 @@ __global__ void __launch_bounds__(kThreads) k_rotate(OuterArgs a, double* X, int
 }
 
 void outer_rotate(const OuterArgs& a, double* X, int kk, int c0, int ncol, double* vout, cudaStream_t s) {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * ((size_t)kMMax * kRotRows + (size_t)kMMax * (kMMax + 1))));
+    static PerDeviceOnce once;
+    once([] {
+        return cudaFuncSetAttribute(k_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(sizeof(double) * ((size_t)kMMax * kRotRows + (size_t)kMMax * (kMMax + 1))));
     });
     const size_t smem = sizeof(double) * ((size_t)kk * kRotRows + (size_t)kk * (ncol + 1));
     k_rotate<<<wave_of((const void*)k_rotate, smem, a.ts_blocks), kThreads, smem, s>>>(a, X, kk, c0, ncol, vout);
