@@ -217,6 +217,16 @@ ISIRA_API isira_status isira_eigpairs(isira_handle h, double* h_eigvals, double*
 /* Counters of the handle (see isira_stats). */
 ISIRA_API isira_status isira_get_stats(isira_handle h, isira_stats* out);
 
+/* How an inner solve of the given precision and deflation rank c (0 <= c <= 31) runs on this handle.  The choice
+ * depends on the graph, the options, the precision and the rank only. */
+typedef struct {
+    int one_launch_ctas;      /* CTAs of the one-launch solve (see isira_opts.inner_graph); 0: launches per iteration */
+    int staged;               /* 1: its CTAs gather from a copy of the vector in their shared memory */
+    int renumbered;           /* 1: the handle's rows are numbered by clusters of the multilevel hierarchy */
+} isira_route;
+
+ISIRA_API isira_status isira_inner_route(isira_handle h, int precision, int c, isira_route* out);
+
 /* 1 = time every phase-1 launch with CUDA events during later solves (adds events between launches; the
  * one-launch solve of a small graph reads the GPU's timer instead; results unchanged), 0 = off. */
 ISIRA_API isira_status isira_set_profiling(isira_handle h, int on);

@@ -31,7 +31,7 @@ ISIRA_MIXED = 1
 
 EXPORTED = ["isira_default_opts", "isira_error_string", "isira_create", "isira_create_weighted", "isira_solve",
             "isira_eigpairs",
-            "isira_get_stats", "isira_set_profiling", "isira_destroy", "isira_apply_operator",
+            "isira_get_stats", "isira_inner_route", "isira_set_profiling", "isira_destroy", "isira_apply_operator",
             "isira_inner_solve", "isira_sym_eig", "isira_sym_eig_warm", "isira_residual_history", "isira_apply_operator_noalloc", "isira_batch_create",
             "isira_precond_apply",
             "isira_batch_solve", "isira_batch_status", "isira_batch_eigpairs", "isira_batch_get_stats",
@@ -72,6 +72,10 @@ class isira_stats(C.Structure):
         return out
 
 
+class isira_route(C.Structure):
+    _fields_ = [("one_launch_ctas", C.c_int), ("staged", C.c_int), ("renumbered", C.c_int)]
+
+
 def _load() -> C.CDLL:
     if not os.path.exists(LIB_PATH):
         raise ImportError(f"libisira.so is not built ({LIB_PATH}); run __graft_entry__.build() or "
@@ -92,6 +96,8 @@ def _load() -> C.CDLL:
     lib.isira_eigpairs.restype = I
     lib.isira_get_stats.argtypes = [P, C.POINTER(isira_stats)]
     lib.isira_get_stats.restype = I
+    lib.isira_inner_route.argtypes = [P, I, I, C.POINTER(isira_route)]
+    lib.isira_inner_route.restype = I
     lib.isira_set_profiling.argtypes = [P, I]
     lib.isira_set_profiling.restype = I
     lib.isira_destroy.argtypes = [P]
@@ -285,6 +291,12 @@ class Solver:
         st = isira_stats()
         check(lib.isira_get_stats(self.h, C.byref(st)), "isira_get_stats")
         return st.as_dict()
+
+    def inner_route(self, c: int = 0, precision: int = ISIRA_MIXED) -> dict:
+        """How an inner solve of this precision and deflation rank runs (isira_inner_route)."""
+        r = isira_route()
+        check(lib.isira_inner_route(self.h, int(precision), int(c), C.byref(r)), "isira_inner_route")
+        return {f: getattr(r, f) for f, _ in r._fields_}
 
     def set_profiling(self, on: bool):
         check(lib.isira_set_profiling(self.h, int(bool(on))), "isira_set_profiling")

@@ -322,6 +322,14 @@ template <typename T> const ClusterPlan& cluster_of(isira_handle h);
 template <> const ClusterPlan& cluster_of<float>(isira_handle h) { return h->cl_f; }
 template <> const ClusterPlan& cluster_of<double>(isira_handle h) { return h->cl_d; }
 
+// the one-launch plan of a diagonally preconditioned inner solve of rank c, or null: launches per iteration
+template <typename T>
+const ClusterPlan* one_launch(isira_handle h, int c) {
+    (void)c;
+    const ClusterPlan& p = cluster_of<T>(h);
+    return h->opts.inner_graph && p.ctas > 0 ? &p : nullptr;
+}
+
 // Counters of the inner solve in flight, once the stream has been synchronised.
 void finish_inner(isira_handle h) {
     if (!h->pending_inner_stats) return;
@@ -360,9 +368,8 @@ int run_inner(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* 
         gram_setup<T>(a, h->Gm, h->Cinv, h->partial, s);
         h->stats.kernel_launches += 1;
     }
-    const ClusterPlan& plan = cluster_of<T>(h);
-    if (plan.ctas > 0 && h->opts.inner_graph) {
-        ck(cluster_minres<T>(a, plan, R, rnorm_dev, h->Z, h->profiling != 0, s));
+    if (const ClusterPlan* plan = one_launch<T>(h, c)) {
+        ck(cluster_minres<T>(a, *plan, R, rnorm_dev, h->Z, h->profiling != 0, s));
         h->stats.kernel_launches += 1;
         h->stats.inner_solves += 1;
         h->pending_inner_stats = -1;
@@ -1405,6 +1412,17 @@ isira_status isira_get_stats(isira_handle h, isira_stats* out) {
     }
     h->stats.hub_timeouts = to;
     *out = h->stats;
+    return ISIRA_OK;
+}
+
+isira_status isira_inner_route(isira_handle h, int precision, int c, isira_route* out) {
+    if (!h || !out || c < 0 || c >= kCMax || (precision != ISIRA_FP64 && precision != ISIRA_MIXED))
+        return ISIRA_ERR_INVALID_ARG;
+    const ClusterPlan* p = nullptr;
+    if (!h->use_ml) p = precision == ISIRA_MIXED ? one_launch<float>(h, c) : one_launch<double>(h, c);
+    out->one_launch_ctas = p ? p->ctas : 0;
+    out->staged = p ? p->staged : 0;
+    out->renumbered = h->visit.empty() ? 0 : 1;
     return ISIRA_OK;
 }
 
