@@ -451,17 +451,20 @@ int run_inner(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* 
 // Takes the solver's copy of the graph (all rows sliced) into the numbering `place` (new -> old of the
 // present one).  Called in create before anything but the hierarchy depends on the numbering: rows keep their
 // entries' order and the clusters their members', so operator and V-cycle give the same sums as before.
-// False, with nothing changed, if there is no memory for the second copy.
+// Every buffer of the new copy, the sliced one and its scratch included, is taken before anything of the
+// handle changes: false, with nothing changed, if there is no memory for it.
 bool relocate(isira_handle h, std::vector<int32_t> place) {
     cudaStream_t s = h->stream;
     const int64_t n = h->n;
-    int32_t *order = nullptr, *perm2 = nullptr, *inv2 = nullptr;
-    int64_t* rp2 = nullptr;
-    int32_t* ci2 = nullptr;
-    double* w2 = nullptr;
+    RowSched& rs = h->rs;
+    int32_t *order = nullptr, *perm2 = nullptr, *inv2 = nullptr, *ci2 = nullptr, *sell_ci2 = nullptr;
+    int64_t *rp2 = nullptr, *sell_off2 = nullptr;
+    double *w2 = nullptr, *sell_wd2 = nullptr;
+    float* sell_wf2 = nullptr;
+    int64_t total2 = 0;
     const size_t nnz_pad = ((size_t)h->nnz + 3) / 4 * 4;
     auto drop = [&] {
-        void* p[] = {order, perm2, inv2, rp2, ci2, w2};
+        void* p[] = {order, perm2, inv2, rp2, ci2, w2, sell_off2, sell_ci2, sell_wd2, sell_wf2};
         for (void* q : p)
             if (q) cudaFree(q);
     };
@@ -472,9 +475,12 @@ bool relocate(isira_handle h, std::vector<int32_t> place) {
         ck(cudaMalloc(&rp2, sizeof(int64_t) * (size_t)(n + 1)));
         ck(cudaMalloc(&ci2, sizeof(int32_t) * nnz_pad));
         if (h->own_w) ck(cudaMalloc(&w2, sizeof(double) * (size_t)h->nnz));
+        ck(cudaMalloc(&sell_off2, sizeof(int64_t) * (size_t)(rs.n_slices + 1)));
         ck(cudaMemcpyAsync(order, place.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, s));
         ck(cudaMemsetAsync(ci2 + h->nnz, 0, sizeof(int32_t) * (nnz_pad - (size_t)h->nnz), s));
         ck(build_permuted_graph(h->own_rp, h->own_ci, h->own_w, n, h->perm, order, rp2, ci2, w2, perm2, inv2, s));
+        ck(build_sell(rp2, ci2, w2, n, 0, rs.n_slices, sell_off2, &sell_ci2, w2 ? &sell_wd2 : nullptr, &total2, s));
+        if (w2) ck(cudaMalloc(&sell_wf2, sizeof(float) * (size_t)std::max<int64_t>(1, total2)));
     } catch (const CudaError& e) {
         drop();
         if (e.e != cudaErrorMemoryAllocation) throw;
@@ -487,34 +493,28 @@ bool relocate(isira_handle h, std::vector<int32_t> place) {
     std::swap(h->perm, perm2);
     std::swap(h->inv, inv2);
     std::swap(h->visit_dev, order);
+    std::swap(h->sell_off, sell_off2);
+    std::swap(h->sell_ci, sell_ci2);
+    std::swap(h->sell_wd, sell_wd2);
+    std::swap(h->sell_wf, sell_wf2);
+    h->sell_total = total2;
     drop();                                               // the old arrays
     int64_t t = 0;
     while (place[(size_t)t] != h->trim) ++t;
     h->trim = t;
     h->visit = std::move(place);
-    RowSched& rs = h->rs;
     rs.rp = h->rp = h->own_rp;
     rs.ci = h->ci = h->own_ci;
+    rs.sell_off = h->sell_off;
+    rs.sell_ci = h->sell_ci;
     setup_deg32(h->own_rp, n, h->ld, h->deg32, s);
     if (h->own_w) {
         rs.wd = h->own_w;
         setup_weighted(h->own_rp, h->own_w, n, h->ld, h->nnz, h->degwd, h->degwf, h->wf, s);
-    }
-    void* sell[] = {h->sell_ci, h->sell_wd, h->sell_wf};
-    for (void* p : sell)
-        if (p) cudaFree(p);
-    h->sell_ci = nullptr;
-    h->sell_wd = nullptr;
-    h->sell_wf = nullptr;
-    ck(build_sell(h->own_rp, h->own_ci, h->own_w, n, 0, rs.n_slices, h->sell_off, &h->sell_ci,
-                  h->own_w ? &h->sell_wd : nullptr, &h->sell_total, s));
-    if (h->own_w) {
-        ck(cudaMalloc(&h->sell_wf, sizeof(float) * (size_t)std::max<int64_t>(1, h->sell_total)));
         copy_cast<float>(h->sell_wd, h->sell_wf, h->sell_total, s);
         rs.swd = h->sell_wd;
         rs.swf = h->sell_wf;
     }
-    rs.sell_ci = h->sell_ci;
     unsigned long long* scr = reinterpret_cast<unsigned long long*>(h->dscratch);
     cluster_plan<float>(rs, h->sell_total, scr, s, &h->cl_f);
     cluster_plan<double>(rs, h->sell_total, scr, s, &h->cl_d);
