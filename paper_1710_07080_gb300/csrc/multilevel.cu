@@ -677,13 +677,15 @@ cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci
             }
         }
         std::vector<double> inv;
-        if (!dense_inverse(levels[L - 1], L == 1 ? skip_old : -1, inv)) return cudaErrorInvalidValue;
+        if (!dense_inverse(levels[L - 1], L == 1 ? skip_old : -1, inv)) throw CudaFailure{cudaErrorInvalidValue};
         upload<T>(&H.inv, inv);
         H.n_coarse = levels[L - 1].n;
         CUDA_OK(cudaStreamSynchronize(s));
     } catch (CudaFailure& f) {
+        ml_free<T>(H);                       // nothing half built stays: the next call builds again
         return f.e;
     } catch (std::bad_alloc&) {
+        ml_free<T>(H);
         return cudaErrorMemoryAllocation;
     }
     return cudaSuccess;

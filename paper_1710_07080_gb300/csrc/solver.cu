@@ -159,8 +159,11 @@ void alloc_inner(isira_handle h, InnerBuffers<T>& b) {
     if (b.base) return;
     // 7 MINRES vectors, plus the reciprocal preconditioner diagonal in FP64 mode
     const int nvec = sizeof(T) == sizeof(double) ? 8 : 7;
-    ck(cudaMalloc(&b.base, sizeof(T) * (size_t)h->ld * nvec));
-    ck(cudaMalloc(&b.st, sizeof(InnerState<T>)));
+    // base last: a call that found no memory for the one or the other is followed by one that asks again
+    T* base = nullptr;
+    if (!b.st) ck(cudaMalloc(&b.st, sizeof(InnerState<T>)));
+    ck(cudaMalloc(&base, sizeof(T) * (size_t)h->ld * nvec));
+    b.base = base;
     ck(cudaMemsetAsync(b.base, 0, sizeof(T) * (size_t)h->ld * nvec, h->stream));
     ck(cudaMemsetAsync(b.st, 0, sizeof(InnerState<T>), h->stream));
 }
@@ -945,6 +948,7 @@ void free_handle(isira_handle h) {
 }
 
 isira_status map_cuda(cudaError_t e) {
+    (void)cudaGetLastError();      // reported by this call: the next one must not meet it again
     if (e == cudaErrorMemoryAllocation) return ISIRA_ERR_OOM;
     return ISIRA_ERR_CUDA;
 }

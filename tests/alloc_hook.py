@@ -16,7 +16,7 @@ ALLOC = """
 static long long calls = 0, refuse = -1, sizes[4096];
 cudaError_t test_malloc(void** p, size_t bytes) {
     if (calls < 4096) sizes[calls] = (long long)bytes;
-    if (calls++ == refuse) return cudaErrorMemoryAllocation;
+    if (calls++ == refuse) return cudaMalloc(p, (size_t)1 << 60);      // refused by the runtime, its last error set
     return cudaMalloc(p, bytes);
 }
 #define API extern "C" __attribute__((visibility("default")))
