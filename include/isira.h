@@ -76,7 +76,9 @@ typedef struct {
     uint64_t seed;        /* SplitMix64 seed of replacement vectors after an orthogonalisation
                              breakdown and of the default start vector */
     int spmv_lanes;       /* lanes per row of the light-row SpMV (1,2,4,8,16,32); <= 0: autotune */
-    int inner_chunk;      /* chunked mode: inner iterations launched between convergence checks; <= 0: 16 */
+    int inner_chunk;      /* chunked mode (inner_graph = 0; solves that are profiled with CUDA events; single inner
+                             solves with blocking_sync = 1): inner iterations launched between convergence
+                             checks; <= 0: 16 */
     int inner_graph;      /* 1: each inner solve is one CUDA-graph launch whose WHILE node repeats the
                              iteration until the device-side stopping test fires (no host round trip),
                              or, on small graphs without rows above 64 neighbours and with the diagonal
@@ -139,7 +141,10 @@ typedef struct {
     int restarts, breakdowns;
     long long inner_iters;    /* total MINRES iterations */
     long long inner_solves;
-    long long spmv_launches;  /* launches of the inner operator's gather kernel (phase 1) */
+    long long spmv_launches;  /* launches of the inner operator's gather kernel (phase 1).  This and
+                                 kernel_launches leave out launches that find the solve stopped and
+                                 return at once, but for chunked mode, which counts whole chunks; the
+                                 one-launch solve of a small graph counts its iterations here */
     double solve_ms;          /* host wall time of the last isira_solve */
     double inner_phase1_ms;   /* summed device time of the phase-1 gather launches (profiling on only); in the
                                  one-launch solve of a small graph, and with the multilevel preconditioner on

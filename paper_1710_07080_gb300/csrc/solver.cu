@@ -264,9 +264,8 @@ int nc_bucket(int c) { return c == 0 ? 0 : (c <= 8 ? 1 : (c <= 12 ? 2 : (c <= 16
 // iteration count and its stopping flag to mapped host memory, and the host keeps `ahead` iterations
 // enqueued beyond the count it sees, so at most that many run empty after the stop (a check after
 // chunks of 16 left 8 on average, of 3 or 16 launches each).  Ends with the stream synchronised.
-// Returns the number of iterations enqueued.
 template <typename F>
-int run_ahead(isira_handle h, int max_it, int ahead, F launch) {
+void run_ahead(isira_handle h, int max_it, int ahead, F launch) {
     volatile HostStatus* st = hst(h);
     int launched = 0;
     for (long long polls = 0; !st->inner_done && launched < max_it;) {
@@ -281,7 +280,17 @@ int run_ahead(isira_handle h, int max_it, int ahead, F launch) {
         }
     }
     sync(h);
-    return launched;
+}
+
+// Counters of such a solve.  How many launches ran empty after the stop depends on timing: they are not
+// counted, as those of a WHILE body after the stop are not.  Returns the iteration count.
+int count_ahead(isira_handle h, int launches_per_iteration) {
+    const int its = hst(h)->inner_iters;
+    h->stats.spmv_launches += its;
+    h->stats.kernel_launches += (long long)launches_per_iteration * its + 1;
+    h->stats.inner_solves += 1;
+    h->stats.inner_iters += its;
+    return its;
 }
 
 // before the launches of a solve that run_ahead drives (the stream holds no earlier work of the handle)
@@ -385,16 +394,12 @@ int run_inner(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const T* 
     inner_phase2<T>(a, 1, s);
     h->stats.kernel_launches += 2;
     if (ahead) {
-        const int nl = run_ahead(h, max_it, 4, [&] {
+        run_ahead(h, max_it, 4, [&] {
             inner_phase1<T>(a, h->lanes, s);
             inner_phase2<T>(a, 0, s);
         });
         inner_finalize_to<T>(a, h->Z, s);
-        h->stats.spmv_launches += nl;
-        h->stats.kernel_launches += 3 * nl + 1;
-        h->stats.inner_solves += 1;
-        h->stats.inner_iters += hst(h)->inner_iters;
-        return hst(h)->inner_iters;
+        return count_ahead(h, 3);
     }
     if (allow_graph && h->opts.inner_graph && !h->profiling) {
         const int bkt = nc_bucket(c);
@@ -629,13 +634,9 @@ int run_inner_ml(isira_handle h, InnerBuffers<T>& b, double sigma, int c, const 
     const int per_it = ml_launches_per_iteration(b, a);
     h->stats.kernel_launches += per_it - 1;
     if (ahead) {
-        const int nl = run_ahead(h, max_it, 2, [&] { ml_iteration<T>(h, b, a, cudaGraphConditionalHandle{}, 0, s); });
+        run_ahead(h, max_it, 2, [&] { ml_iteration<T>(h, b, a, cudaGraphConditionalHandle{}, 0, s); });
         inner_finalize_to<T>(a, h->Z, s);
-        h->stats.spmv_launches += nl;
-        h->stats.kernel_launches += (long long)per_it * nl + 1;
-        h->stats.inner_solves += 1;
-        h->stats.inner_iters += hst(h)->inner_iters;
-        return hst(h)->inner_iters;
+        return count_ahead(h, per_it);
     }
     if (allow_graph && h->opts.inner_graph && !h->profiling) {
         const int bkt = nc_bucket(c);
