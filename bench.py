@@ -323,6 +323,17 @@ def kernel_bytes(kind, n, Z, c, word, n_long=None, n_slices=None, ml=None):
         struct = 8 * (n + 1) if not n_slices else 8 * (n_long + 1) + 8 * (n_slices + 1)
         return ((21 + 4 * c) * word * n + 8 * n + 2 * (struct + 4 * Z)
                 + 2 * (4 + word) * nnz_c + (16 + 9 * word) * n_c)
+    if kind == "phase2_ml_u":
+        # the same above deflation rank 8, where the gather of x1 stores W x1 and phase 2b is a kernel of its own:
+        # W x1 written and read and x1 read once more
+        return kernel_bytes("phase2_ml_s", n, Z, c, word, n_long, n_slices, ml) + 3 * word * n
+    if kind == "one_launch":
+        # one iteration of the one-launch solve: the Krylov vectors stay in shared memory; indices and gathered
+        # values (Z here: the sliced copy's entries), slice offsets, z written, Vh read by both phases
+        return (4 + word) * Z + 16 * n_slices + word * n + 2 * c * word * n
+    if kind == "one_launch_staged":
+        # the gathers read shared memory; every CTA (ml here: their number) copies z
+        return 4 * Z + 16 * n_slices + word * n + ml * word * n + 2 * c * word * n
     if kind == "gather":
         struct = 8 * (n + 1) if not n_slices else 8 * (n_long + 1) + 8 * (n_slices + 1)
         return struct + 4 * Z + 2 * word * n
@@ -383,24 +394,57 @@ def hbm_peak():
     return FALLBACK_HBM_GBS, "fallback"
 
 
-def kernel_rooflines(st, n, Z, word, workload, prec_tag):
-    """Per-kernel achieved GB/s from one profiled solve's CUDA-event totals, and the dominant one."""
+def one_launch_rooflines(st, n, word, routes):
+    """The entry of a profiled solve whose inner solves run in one launch (at least at some ranks): one kernel
+    whose vectors live in shared memory, bound by latency and, in FP64, by the FP64 pipe of its SMs.
+    Its traffic goes to L2, so no fraction of the HBM peak is stated."""
+    nl = st["inner_phase1_timed"]
+    c_avg = st["inner_phase1_csum"] / max(1, nl)
+    taken = [c for c, r in enumerate(routes) if r["one_launch_ctas"]]
+    r0 = routes[taken[0]]
+    parts = {kind: st[STAT_OF[kind]] for kind in STAT_OF}
+    total = sum(parts.values())
+    avg_s = total / 1e3 / max(1, nl)
+    n_slices = (n + 31) // 32
+    kind = "one_launch_staged" if r0["staged"] else "one_launch"
+    b = kernel_bytes(kind, n, st["sell_entries"], c_avg, word, 0, n_slices, r0["one_launch_ctas"])
+    name = f"k_minres_cluster (the whole inner solve in one cluster of {r0['one_launch_ctas']} CTAs)"
+    if len(taken) < len(routes):
+        name += (f"; ranks {', '.join(str(c) for c in range(len(routes)) if c not in taken)} take k_phase1_gather_s, "
+                 "k_phase1 and k_phase2, whose time is included")
+    entry = {"kernel": name, "bound": "latency" if word == 4 else "latency and the FP64 pipe of its SMs",
+             "achieved": b / avg_s / 1e9 if avg_s > 0 else None, "peak": None, "unit": "GB/s of L2 traffic",
+             "frac": None, "bytes_per_launch": b, "avg_us": avg_s * 1e6, "launches_timed": nl, "total_ms": total,
+             "avg_deflation_rank": c_avg, "traffic": None, "share_of_inner_kernels": 1.0 if total > 0 else None,
+             "parts_ms": {"gather_and_rows": parts["gather"], "phase1_sums": parts["rows"], "phase2": parts["phase2"]}}
+    return {"one_launch": entry}
+
+
+def kernel_rooflines(st, n, Z, word, workload, prec_tag, routes=()):
+    """Per-kernel achieved GB/s from one profiled solve's CUDA-event totals, and the dominant one.  routes: how
+    an inner solve of deflation rank 0, 1, ... runs (Solver.inner_route)."""
     peak, peak_src = hbm_peak()
+    if any(r["one_launch_ctas"] for r in routes):
+        return one_launch_rooflines(st, n, word, routes), "one_launch", peak_src
     nl = st["inner_phase1_timed"]
     c_avg = st["inner_phase1_csum"] / max(1, nl)
     n_slices = (n - st["n_long_rows"] + 31) // 32 if st.get("sell_entries") else None
     ml = st.get("precond") == 1
     names = KERNEL_NAMES_ML if ml else KERNEL_NAMES
+    ranks = max(1, len(routes))
     out = {}
     for kind in ("gather", "rows", "phase2"):
         ms = st[STAT_OF[kind]]
         avg_s = ms / 1e3 / max(1, nl)
         bkind = kind + "_ml" if ml and kind != "gather" else kind
+        args = (n, Z, c_avg, word, st["n_long_rows"], n_slices, (st.get("ml_coarse_n", 0), st.get("ml_coarse_nnz", 0)))
         if ml and n_slices and not st["n_long_rows"]:
             # every row sliced: phase 1 is one kernel, timed as the gather
             bkind = {"gather": "gather_ml_s", "phase2": "phase2_ml_s"}.get(kind, bkind)
-        b = kernel_bytes(bkind, n, Z, c_avg, word, st["n_long_rows"], n_slices,
-                         (st.get("ml_coarse_n", 0), st.get("ml_coarse_nnz", 0)))
+        b = kernel_bytes(bkind, *args)
+        if bkind == "phase2_ml_s" and ranks > 9:
+            # post-smoothing is fused with the gather up to rank 8; iterations taken as even over the ranks
+            b += (kernel_bytes("phase2_ml_u", *args) - b) * (ranks - 9) / ranks
         ach = b / avg_s / 1e9 if avg_s > 0 else None
         out[kind] = {"kernel": names[kind], "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
                      "frac": ach / peak if ach else None, "bytes_per_launch": b, "avg_us": avg_s * 1e6,
@@ -746,7 +790,8 @@ def main():
     t_stage = time.perf_counter()
     t_oth, st_oth = timed(solvers[other], 1, max(1, min(args.steps, args.cmp_steps)))
     stages["timed_other_precision_s"] = time.perf_counter() - t_stage
-    # kernel timing: one solve per precision with CUDA events around every inner launch (chunked launches)
+    # kernel timing: one solve per precision with CUDA events around every inner launch (chunked launches; the
+    # one-launch solve of a small graph reads the GPU's timer)
     t_stage = time.perf_counter()
     prof = {p: timed(solvers[p], 0, 1, profile=True) for p in (head, other)}
     stages["profiled_solves_s"] = time.perf_counter() - t_stage
@@ -794,10 +839,11 @@ def main():
     word = {"fp64": 8, "mixed": 4}
     kern = {}
     for p in (head, other):
-        kern[p] = kernel_rooflines(prof[p][1][0], n, Z, word[p], args.workload, "f32" if p == "mixed" else "f64")
+        routes = [solvers[p].inner_route(c, P[p]) for c in range(k)]
+        kern[p] = kernel_rooflines(prof[p][1][0], n, Z, word[p], args.workload, "f32" if p == "mixed" else "f64", routes)
     rk, dom, peak_src = kern[head]
     roof = dict(rk[dom])
-    roof.update(peak_source=peak_src, dominant_of="inner-iteration kernels (gather, rows, phase2), by total time",
+    roof.update(peak_source=peak_src, dominant_of=f"inner-iteration kernels ({', '.join(rk)}), by total time",
                 other_kernels={q: {kk: v[kk] for kk in ("kernel", "achieved", "frac", "avg_us", "share_of_inner_kernels")}
                                for q, v in rk.items() if q != dom})
     ro, dom_o, _ = kern[other]
