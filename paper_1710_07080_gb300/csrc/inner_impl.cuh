@@ -1083,19 +1083,19 @@ __global__ void __launch_bounds__(kThreads) k_ml_phase2a(InnerArgs<T> a, int ini
             __syncthreads();
         }
     }
-    if (NE == 0) return;
-    __shared__ T bv[NE > 0 ? NE : 1];
+    if constexpr (NE > 0) {
+        __shared__ T bv[NE], red[NE];
 #pragma unroll
-    for (int q = 0; q < QW; ++q) {
-        const int t = warp + q * kWarps;
-        const T sh = warp_sum(ch[q]);
-        if (lane == 0 && t < NE) bv[t] = t < c ? sh : T(0);
-    }
-    __syncthreads();
-    __shared__ T red[NE > 0 ? NE : 1];
-    if (block_values_arrive<T>(bv, NE, a.partial, a.pstride, a.counter)) {
-        last_block_sum(a.partial, a.pstride, gridDim.x, NE, red, a.counter);
-        for (int t = threadIdx.x; t < c; t += blockDim.x) st->hv[t] = red[t];
+        for (int q = 0; q < QW; ++q) {
+            const int t = warp + q * kWarps;
+            const T sh = warp_sum(ch[q]);
+            if (lane == 0 && t < NE) bv[t] = t < c ? sh : T(0);
+        }
+        __syncthreads();
+        if (block_values_arrive<T>(bv, NE, a.partial, a.pstride, a.counter)) {
+            last_block_sum(a.partial, a.pstride, gridDim.x, NE, red, a.counter);
+            for (int t = threadIdx.x; t < c; t += blockDim.x) st->hv[t] = red[t];
+        }
     }
 }
 

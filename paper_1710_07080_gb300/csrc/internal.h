@@ -28,9 +28,9 @@ struct MlLevel {
     int32_t* rp = nullptr;                    // level >= 1: CSR of the off-diagonal weights
     int32_t* ci = nullptr;
     T* w = nullptr;
-    int32_t* agg = nullptr;                   // vertex -> cluster of the next level (-1: none)
-    int64_t* mrp = nullptr;                   // members of each cluster of the next level
-    int32_t* mem = nullptr;
+    int64_t* mrp = nullptr;                   // members of each cluster of the next level: rows (levels >= 1), or
+    int32_t* mem = nullptr;                   // entries of mem (level 0)
+    int32_t* agg = nullptr;                   // level 0: vertex -> cluster of the next level (-1: none)
     T* b = nullptr;                           // right-hand side of this level (levels >= 1)
     T* x0 = nullptr; T* x1 = nullptr; T* x = nullptr;   // work vectors (levels >= 1: x0 holds D^{-1} b)
 };
@@ -58,8 +58,8 @@ template <typename T> void ml_free(MlHierarchy<T>& H);
 // out = M^{-1} b, one V-cycle; kernels return at once while *done != 0 (done may be null)
 template <typename T>
 void ml_vcycle(MlHierarchy<T>& H, const T* b, T* out, const GatherFn<T>& gather, T omega, T alpha, const int* done,
-               bool x0_ready, bool skip_post0, const int32_t* perm, cudaStream_t s);
-template <typename T> int ml_launches(const MlHierarchy<T>& H, bool x0_ready, bool skip_post0);
+               bool skip_post0, const int32_t* perm, cudaStream_t s);
+template <typename T> int ml_launches(const MlHierarchy<T>& H, bool skip_post0);
 // b and level 0's x0 from the caller's x (perm: the caller's numbering; null: the solver's); nlev >= 2
 template <typename T>
 void ml_stage(MlHierarchy<T>& H, const T* x, const int32_t* perm, T omega, T* b, cudaStream_t s);

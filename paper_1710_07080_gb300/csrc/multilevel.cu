@@ -28,7 +28,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <numeric>
 #include <vector>
 
@@ -206,15 +205,6 @@ static bool dense_inverse(const HostLevel& A, int64_t skip, std::vector<double>&
 }
 
 // ------------------------------------------------------------------ device kernels of the V-cycle
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_ml_scale(const T* __restrict__ b, const T* __restrict__ dinv, T om,
-                                                       int64_t n, int64_t skip, T* __restrict__ x,
-                                                       const int* __restrict__ done) {
-    if (done && *done) return;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = i == skip ? T(0) : om * b[i] * dinv[i];
-}
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_ml_stage(const T* __restrict__ x, const int32_t* __restrict__ perm,
@@ -659,21 +649,25 @@ cudaError_t ml_build(MlHierarchy<T>& H, const int64_t* d_rp, const int32_t* d_ci
             CUDA_OK(cudaMemsetAsync(D.x0, 0, sizeof(T) * nv, s));
             CUDA_OK(cudaMemsetAsync(D.x1, 0, sizeof(T) * nv, s));
             if (l + 1 < L) {
+                // cluster boundaries; the coarse rows are ordered by cluster, level 0's are not: it also takes
+                // the cluster of every row and the members of every cluster
                 const std::vector<int32_t>& agg = aggs[l];
-                std::vector<int32_t> agg_pad(nv, -1);
-                for (int64_t i = 0; i < (int64_t)agg.size(); ++i) agg_pad[place_of(i)] = agg[i];
-                upload_i<int32_t>(&D.agg, agg_pad);
                 const int64_t nc = levels[l + 1].n;
                 std::vector<int64_t> mrp(nc + 1, 0);
                 for (int32_t I : agg)
                     if (I >= 0) mrp[I + 1]++;
                 for (int64_t I = 0; I < nc; ++I) mrp[I + 1] += mrp[I];
-                std::vector<int32_t> mem(mrp[nc]);
-                std::vector<int64_t> fill(mrp.begin(), mrp.end() - 1);
-                for (int64_t i = 0; i < (int64_t)agg.size(); ++i)
-                    if (agg[i] >= 0) mem[fill[agg[i]]++] = (int32_t)place_of(i);   // members in the old order
                 upload_i<int64_t>(&D.mrp, mrp);
-                upload_i<int32_t>(&D.mem, mem);
+                if (l == 0) {
+                    std::vector<int32_t> agg_pad(nv, -1), mem(mrp[nc]);
+                    std::vector<int64_t> fill(mrp.begin(), mrp.end() - 1);
+                    for (int64_t i = 0; i < (int64_t)agg.size(); ++i) {
+                        agg_pad[place_of(i)] = agg[i];
+                        if (agg[i] >= 0) mem[fill[agg[i]]++] = (int32_t)place_of(i);   // members in the old order
+                    }
+                    upload_i<int32_t>(&D.agg, agg_pad);
+                    upload_i<int32_t>(&D.mem, mem);
+                }
             }
         }
         std::vector<double> inv;
@@ -723,12 +717,12 @@ constexpr int kMlLanes = 4;          // lanes per coarse CSR row
 
 // out = M^{-1} b (b on level 0, n-space, the trimmed entry ignored; out may alias nothing else).
 // gather(x, res, g) must compute g = W x (+ (1 - omega) res, if res is not null) for level 0.
-// x0_ready: level 0's x0 = w D^{-1} b is already in H.lev[0].x0 (written by the caller's kernel).
+// Level 0's x0 = w D^{-1} b is in H.lev[0].x0 already (nlev >= 2; written by the caller's kernel).
 // skip_post0 (nlev >= 2): stop before the gather of x1 (H.lev[0].x1) that the caller's next kernels make, with
 // level 0's post-smoothing (out is then not written).
 template <typename T>
 void ml_vcycle(MlHierarchy<T>& H, const T* b, T* out, const GatherFn<T>& gather, T omega, T alpha, const int* done,
-               bool x0_ready, bool skip_post0, const int32_t* perm, cudaStream_t s) {
+               bool skip_post0, const int32_t* perm, cudaStream_t s) {
     const int L = H.nlev;
     MlLevel<T>& F = H.lev[0];
     if (L == 1) {
@@ -736,8 +730,7 @@ void ml_vcycle(MlHierarchy<T>& H, const T* b, T* out, const GatherFn<T>& gather,
                                                              nullptr, done);
         return;
     }
-    // level 0 down: x0 = w D^{-1} b, the residual (1 - w) b + W x0 in the solver's gather, restricted
-    if (!x0_ready) k_ml_scale<T><<<ml_grid(F.n), kThreads, 0, s>>>(b, F.dinv, omega, F.n, H.skip, F.x0, done);
+    // level 0 down: the residual (1 - w) b + W x0 in the solver's gather, restricted
     gather(F.x0, b, F.x, s);
     {
         MlLevel<T>& C = H.lev[1];
@@ -776,9 +769,9 @@ void ml_vcycle(MlHierarchy<T>& H, const T* b, T* out, const GatherFn<T>& gather,
 
 // launches of one call (without the caller's gather of x1 when skip_post0)
 template <typename T>
-int ml_launches(const MlHierarchy<T>& H, bool x0_ready, bool skip_post0) {
+int ml_launches(const MlHierarchy<T>& H, bool skip_post0) {
     if (H.nlev <= 1) return 1;
-    return (x0_ready ? 0 : 1) + 2 + 2 * (H.nlev - 2) + 1 + 1 + (skip_post0 ? 0 : 2);
+    return 2 + 2 * (H.nlev - 2) + 1 + 1 + (skip_post0 ? 0 : 2);
 }
 
 // b = x (the caller's vector and numbering) and level 0's x0 = w D^{-1} b
@@ -794,9 +787,9 @@ void ml_stage(MlHierarchy<T>& H, const T* x, const int32_t* perm, T omega, T* b,
                                      cudaStream_t);                                                          \
     template void ml_free<T>(MlHierarchy<T>&);                                                               \
     template void ml_vcycle<T>(MlHierarchy<T>&, const T*, T*, const GatherFn<T>&, T, T, const int*, bool,     \
-                               bool, const int32_t*, cudaStream_t);                                          \
+                               const int32_t*, cudaStream_t);                                                \
     template void ml_stage<T>(MlHierarchy<T>&, const T*, const int32_t*, T, T*, cudaStream_t);               \
-    template int ml_launches<T>(const MlHierarchy<T>&, bool, bool);
+    template int ml_launches<T>(const MlHierarchy<T>&, bool);
 ISIRA_INSTANTIATE_ML(float)
 ISIRA_INSTANTIATE_ML(double)
 

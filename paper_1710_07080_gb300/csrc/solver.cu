@@ -569,7 +569,7 @@ void ml_second_phase(isira_handle h, InnerBuffers<T>& b, const InnerArgs<T>& a, 
     ml_phase2a<T>(a, init, s);
     ml_project<T>(a, init, s);
     ml_vcycle<T>(b.H, a.c > 0 ? a.rin : a.rcur, a.wv, ml_gather<T>(h, a, done), (T)kMlOmega, ml_alpha<T>(h), done,
-                 a.ml_x0 != nullptr, a.ml_fuse_post != 0, nullptr, s);
+                 a.ml_fuse_post != 0, nullptr, s);
     ml_finish_cycle<T>(a, init, h->lanes, cond, has_cond, s);
 }
 
@@ -608,7 +608,7 @@ cudaGraphExec_t build_ml_graph(isira_handle h, InnerBuffers<T>& b, const InnerAr
 template <typename T>
 int ml_launches_per_iteration(const InnerBuffers<T>& b, const InnerArgs<T>& a) {
     const bool multi = b.H.nlev >= 2, fused = ml_post_fused(a);
-    return (slices_only(a.rs) ? 1 : 2) + 1 + (a.c > 0 ? 1 : 0) + ml_launches(b.H, multi, multi) +
+    return (slices_only(a.rs) ? 1 : 2) + 1 + (a.c > 0 ? 1 : 0) + ml_launches(b.H, multi) +
            (fused ? 1 : multi ? 2 : 1) + (fused && a.c == 0 ? 0 : 1);
 }
 
@@ -1010,12 +1010,12 @@ void precond_apply_t(isira_handle h, InnerBuffers<T>& b, const T* d_x, T* d_y) {
     if (b.H.nlev >= 2) {
         // the caller's numbering is left and met again inside the cycle's own first and last kernels
         ml_stage<T>(b.H, d_x, h->perm, (T)kMlOmega, a.rcur, s);
-        ml_vcycle<T>(b.H, a.rcur, d_y, ml_gather<T>(h, a, nullptr), (T)kMlOmega, ml_alpha<T>(h), nullptr, true, false,
+        ml_vcycle<T>(b.H, a.rcur, d_y, ml_gather<T>(h, a, nullptr), (T)kMlOmega, ml_alpha<T>(h), nullptr, false,
                      h->perm, s);
     } else {
         if (h->perm) to_internal<T>(d_x, h->perm, h->n, a.rcur, s);
         else ck(cudaMemcpyAsync(a.rcur, d_x, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
-        ml_vcycle<T>(b.H, a.rcur, a.wv, ml_gather<T>(h, a, nullptr), (T)kMlOmega, ml_alpha<T>(h), nullptr, false, false,
+        ml_vcycle<T>(b.H, a.rcur, a.wv, ml_gather<T>(h, a, nullptr), (T)kMlOmega, ml_alpha<T>(h), nullptr, false,
                      nullptr, s);
         if (h->perm) to_external<T>(a.wv, h->perm, h->n, d_y, s);
         else ck(cudaMemcpyAsync(d_y, a.wv, sizeof(T) * h->n, cudaMemcpyDeviceToDevice, s));
