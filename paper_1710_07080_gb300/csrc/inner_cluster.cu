@@ -542,22 +542,44 @@ __global__ void __launch_bounds__(kThreads) k_sell_lines(const int32_t* __restri
     if (lane == 0 && cnt) atomicAdd(out, cnt);
 }
 
-// Which graphs take this path, and how (GB300, per iteration at deflation rank 0 / 8, one launch against
-// three).  The choice depends on the graph and the precision alone, so a graph gives the same bits
-// alone and in a batch.
+// Microseconds that an FP64 iteration takes in one launch and in three, fitted to the measurements below: 16 SMs
+// issue in one launch what 152 issue in three, so rows, columns (rounds of eight, one warp each) and entries
+// cost more there, and the launches cost a constant.
+static bool fp64_one_launch_pays(int64_t n, int64_t entries, bool weighted, int c) {
+    const double kn = 1e-3 * (double)n, ke = 1e-3 * (double)entries;
+    const double rounds = c <= 8 ? c / 8.0 : (double)((c + 7) / 8);
+    const double one = 4.0 + (c > 0 ? 3.0 : 0.0) + 0.17 * c + 0.15 * rounds + kn * (0.36 + 0.055 * c + 0.21 * rounds) +
+                       ke * (weighted ? 0.041 : 0.032);
+    const double three = 26.5 + 0.007 * ke + (c > 0 ? 9.2 + 0.55 * std::min(c, 8) + 1.28 * std::max(c - 8, 0) : 0.0);
+    return one <= three;
+}
+
+// Which solves take this path, and how.  The choice depends on the graph, the precision and the deflation rank
+// alone, so a graph gives the same bits alone and in a batch.  Times are us per iteration on GB300, one launch
+// against three.
 //  * All rows sliced (no row above 64 neighbours): a long row would need its own split over the warps.
-//  * FP32 up to 80,000 rows, where the ten vectors fill the shared memory of 16 CTAs: 2-D grids of 9,856 /
-//    30,600 / 78,400 vertices 3.5 / 7.6, 5.2 / 11.8, 8.2 / 19.7 us against 19 / 28, 21 / 29, 21 / 31 us.  A random graph is bound
-//    by the lines its gathers touch, one per cycle and SM (ER of 40,000: 14.5 / 21.6 us against 22.6 / 33 us),
-//    so beyond kClusterLines lines a CTA the whole GPU is the better place.
-//  * FP64 up to 30,720 rows: 16 SMs issue the FP64 instructions of 152, so the line is where that costs what
-//    the launches did (grids of 9,856 / 30,600 vertices: 9.3 / 19.7 and 18.3 / 42.7 us against 27 / 40 and 29 / 44 us;
-//    ER of 40,000: 34 / 64 against 32 / 46 us).
-//    (The launches' times are those with one iteration a turn of the WHILE node; four take 2 to 3 us off.)
+//  * FP32 up to 80,000 rows, where the ten vectors fill the shared memory of 16 CTAs.  2-D grids of 19,881 /
+//    40,000 / 77,841 vertices at rank 0: 5.0 / 6.3 / 8.7 against 18.5 / 19.4 / 20.5; rank 31: 19 / 28 / 44 against
+//    48 / 51 / 53.  A random graph is bound by the lines its gathers touch, one per cycle and SM (ER of 39,984:
+//    14.8 against 21.7, of 55,986: 19.2 against 22.1), so beyond kClusterLines lines a CTA the whole GPU is the
+//    better place.
+//  * FP32 with more than 196 KB of shared memory a CTA (above 71,168 rows): the L1 that is left no longer holds
+//    what the gathers of a line-heavy graph reuse (Watts-Strogatz of 68,000 / 72,000 / 79,900 at rank 0: 14.3 /
+//    20.6 / 22.1 against 22.5; rank 8: 24.3 / 30.9 / 33.0 against 31.7; rank 24: 38.7 / 45.8 / 49.1 against 45.1).
+//    Above kClusterLinesTight lines it is taken up to rank 8 only; a grid of 77,841 (1,263 lines) at all.
+//  * FP64 up to 30,720 rows, at the ranks where fp64_one_launch_pays: rank 0 / 8 / 16 / 31, grid of 7,921: 8.2 /
+//    17.0 / 23.9 / 36.8 against 26.6 / 39.0 / 49.2 / 67.6; of 19,881: 13.8 / 30.6 / 45.2 / 71.9 against 26.7 / 40.9 /
+//    49.8 / 69.7; of 29,929: 19.0 / 43.0 / 64.2 / 103.8 against 26.7 / 41.0 / 50.2 / 70.6.  Entries count too: of
+//    20,000 rows, 800,000 entries at rank 0: 33.0 against 31.1.  The fit's choice is at most 4 % from the
+//    better path over the 29 graphs that were measured (4,000 to 30,000 rows, 4 to 40 entries a row, with
+//    and without weights, ranks 0 to 31).
 //  * CTAs: enough for 256 rows each in FP32 (latency) and 64 in FP64 (its narrow pipe), 16 at most.
 //  * Staging copies z_k whole into every CTA's shared memory each iteration and gathers from there: it pays
 //    in FP32 when the gathers touch more lines than the copy moves (ER of 12,339: 4.7 us against 6.6 us; grid of
 //    9,856: 3.5 us staged, 3.3 us not); in FP64 the gather hides behind the FP64 pipe (ER of 12,339: 15.5 staged, 14.1 not).
+constexpr int64_t kClusterLinesTight = 8000;
+constexpr int kL1Step = 196 * 1024;         // shared memory beyond which the L1 falls to its smallest size
+
 template <typename T>
 void cluster_plan(const RowSched& rs, int64_t sell_total, unsigned long long* scratch, cudaStream_t s, ClusterPlan* out) {
     *out = ClusterPlan{};
@@ -572,6 +594,7 @@ void cluster_plan(const RowSched& rs, int64_t sell_total, unsigned long long* sc
     p.threads = std::min(ClThreads<T>::value, std::max(128, nsl * 32));
     p.smem = (int)sizeof(T) * kClVecs * p.cap;
     p.staged = 0;
+    p.ranks = ~0u;
     int dev = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
@@ -591,6 +614,12 @@ void cluster_plan(const RowSched& rs, int64_t sell_total, unsigned long long* sc
             p.staged = 1;
             p.smem += (int)zbytes;
         }
+        if (!p.staged && p.smem + (int)sizeof(ClShared<T>) + 1024 > kL1Step && per_cta > kClusterLinesTight)
+            p.ranks = (1u << 9) - 1;
+    } else {
+        p.ranks = 0;
+        for (int c = 0; c < kCMax; ++c)
+            if (fp64_one_launch_pays(rs.n, sell_total, rs.swd != nullptr, c)) p.ranks |= 1u << c;
     }
     if (cudaFuncSetAttribute(k_minres_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess ||
         cudaFuncSetAttribute(k_minres_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {

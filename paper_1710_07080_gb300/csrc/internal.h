@@ -169,8 +169,10 @@ struct ClusterPlan {
     int threads = 0, cap = 0;   // threads and row slots per CTA
     int staged = 0;             // every CTA copies z_k whole into its shared memory and gathers from there
     int smem = 0;               // dynamic shared memory per CTA
+    uint32_t ranks = 0;         // bit c: an inner solve of deflation rank c takes this path
 };
 constexpr int64_t kClusterRows32 = 80000, kClusterRows64 = 30720, kClusterLines = 28000;
+static_assert(kCMax <= 32, "a bit for every deflation rank");
 constexpr int kClusterRowsPerCta32 = 256, kClusterRowsPerCta64 = 64;
 // scratch: 8 device bytes; synchronises s
 template <typename T>

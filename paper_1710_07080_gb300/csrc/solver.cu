@@ -337,9 +337,8 @@ template <> const ClusterPlan& cluster_of<double>(isira_handle h) { return h->cl
 // the one-launch plan of a diagonally preconditioned inner solve of rank c, or null: launches per iteration
 template <typename T>
 const ClusterPlan* one_launch(isira_handle h, int c) {
-    (void)c;
     const ClusterPlan& p = cluster_of<T>(h);
-    return h->opts.inner_graph && p.ctas > 0 ? &p : nullptr;
+    return h->opts.inner_graph && (p.ranks >> c & 1u) ? &p : nullptr;
 }
 
 // Counters of the inner solve in flight, once the stream has been synchronised.

@@ -38,6 +38,22 @@ def test_lines_and_long_rows(make, prec, ctas, staged):
     assert (r["one_launch_ctas"], r["staged"]) == (ctas, staged)
 
 
+@pytest.mark.parametrize("make,prec,ranks", [
+    (lambda: sg.grid2d(63, 63), "fp64", {0: 16, 8: 16, 31: 16}),
+    (lambda: sg.grid2d(126, 126), "fp64", {0: 16, 16: 16, 31: 16}),
+    (lambda: sg.grid2d(173, 173), "fp64", {0: 16, 4: 16, 12: 0, 31: 0}),      # 16 SMs against 152 from here on
+    (lambda: sg.erdos_renyi(30000, 8.0, seed=5), "fp64", {0: 16, 2: 16, 10: 0, 31: 0}),
+    (lambda: sg.watts_strogatz(30000, 20, 0.1, seed=5), "fp64", {0: 0, 8: 0, 31: 0}),
+    (lambda: sg.grid2d(279, 279), "mixed", {0: 16, 31: 16}),
+    (lambda: sg.watts_strogatz(68000, 10, 0.1, seed=6), "mixed", {0: 16, 31: 16}),
+    (lambda: sg.watts_strogatz(79999, 10, 0.1, seed=6), "mixed", {0: 16, 8: 16, 9: 0, 31: 0}),   # little L1 left
+])
+def test_ranks_at_which_one_launch_pays(make, prec, ranks):
+    g = make()
+    for c, ctas in ranks.items():
+        assert route(g, prec, c)["one_launch_ctas"] == ctas, c
+
+
 @pytest.mark.parametrize("opts", [{"inner_graph": 0}, {"precond": 1}, {"reorder": 0}, {"sell": 0}])
 def test_options_that_keep_launches_per_iteration(opts):
     assert route(sg.grid2d(40, 37), "mixed", **opts)["one_launch_ctas"] == 0
