@@ -242,7 +242,9 @@ ISIRA_API void isira_destroy(isira_handle h);
 /* ---------------------------------------------------------------------------------
  * Component entry points: single steps of the method on the handle's graph, used by
  * tests and benchmarks.  Device pointers; results ordered on the handle's stream;
- * each call synchronises before returning.
+ * each call synchronises before returning.  Calls with deflation vectors keep the solver's copy of
+ * them, a buffer of c columns in the call's precision, for the next call if it is at most 1 GiB;
+ * isira_destroy frees it.
  */
 
 /* The implicit operator of Theorem 2.6 (Eq. 2.14) applied in n-space:
@@ -303,8 +305,8 @@ ISIRA_API isira_status isira_sym_eig_warm(int k, int warm_w, const double* d_H, 
  * Batched solves: many independent graphs of uneven size (Algorithm 2 for each graph).
  * Every graph gets its own solver (as isira_create) and its own CUDA stream; a pool of host
  * threads drives the solvers concurrently, largest graphs first, so the kernels of different
- * graphs overlap on the GPU.  Each inner solve is one device-driven CUDA-graph launch
- * (opts->inner_graph).  The caller owns the G CSR graphs (device pointers, as in isira_create)
+ * graphs overlap on the GPU.  Each inner solve is one launch, of the one-launch kernel of small
+ * graphs or of a device-driven CUDA graph (opts->inner_graph).  The caller owns the G CSR graphs (device pointers, as in isira_create)
  * until isira_batch_destroy.
  */
 typedef struct isira_batch_s* isira_batch;
@@ -352,7 +354,8 @@ ISIRA_API void isira_batch_destroy(isira_batch b);
  * Calls no cudaMalloc, cudaFree or allocating routine.  Its cross-CTA partial sums live in a
  * fixed static device array of about 72 KB (held by every GPU that loads the library until the
  * process exits), which limits the deflation rank to c <= 8: larger c returns ISIRA_ERR_LIMIT.
- * All calls share that array: calls whose work overlaps on the GPU race and must be serialised.
+ * All calls share that array: calls whose work overlaps on the GPU race and must be serialised
+ * (a race spoils the racing calls' results, not those of later calls that run alone).
  * The first call on each device, with that device current, looks up the array's device address
  * (cudaGetSymbolAddress); make that first call before any stream capture on the device.
  * Ordered on `stream`; synchronises it before returning. */

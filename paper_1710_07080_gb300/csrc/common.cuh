@@ -662,10 +662,10 @@ __device__ __forceinline__ void for_each_row_gather(const RowSched& S, const T* 
 // The epilogue has two halves: pre(row) loads what it needs of the row's vectors before the gather, so
 // that those loads and the dependent index -> value chains are in flight together, and fin(row, loaded,
 // sum) does the arithmetic.  (Rows up to the next multiple of 32 are loaded: every vector has them.)
-// In FP64 the arithmetic stops at the slice's width: an SM issues an FP64 warp instruction every 16 cycles,
+// In FP64 the arithmetic stops at the slice's width: an SM issues an FP64 warp instruction every 16 to 19 cycles,
 // and a grid's four entries in eight slots cost twice what they need.  The widths are cases of a switch,
 // since the compiler turns short conditional blocks into predicated instructions, and a predicated-off
-// FP64 instruction takes its 16 cycles all the same (2000 passes of width 3: 955 us as a switch, 1249 us as
+// FP64 instruction takes its cycles all the same (2000 passes of width 3: 955 us as a switch, 1249 us as
 // nested conditions, 2489 us at full width).
 template <typename T>
 __device__ __forceinline__ T pass_sum(const T (&v)[8], int r) {

@@ -15,7 +15,7 @@
 //
 // What bounds an iteration: in FP32 the chain of two reductions and two cluster barriers (2.3 us on 20
 // vertices, 3.5 us on a grid of 9,856) and, on random graphs, the lines that the gathers touch; in FP64
-// the FP64 pipe, which issues a warp instruction every 16 cycles on an SM: hence few warps (a warp
+// the FP64 pipe, which issues a warp instruction every 16 to 19 cycles on an SM: hence few warps (a warp
 // reduction costs as much as a row), D z kept instead of D, folded w coefficients, additions only
 // where a slice has entries, and the w / x update placed under the first barrier (9.3 us on the grid of
 // 9,856; 13.3 us before those).
@@ -99,7 +99,7 @@ __device__ __forceinline__ T cl_total(const T* v) {
 }
 
 // Sum of the r gathered values of a pass (r uniform over the warp).  FP64: only the additions that
-// the width needs, since one SM issues an FP64 warp instruction every 16 cycles; FP32: all eight.
+// the width needs, since one SM issues an FP64 warp instruction every 16 to 19 cycles; FP32: all eight.
 template <typename T>
 __device__ __forceinline__ T cl_pass_sum(const T (&v)[8], int r) {
     if constexpr (sizeof(T) == 4) return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));

@@ -838,13 +838,15 @@ constexpr int kTsMaxCols = kMMax + kCMax;
 // Q = [U(:, 0:k) V(:, 0:c)].  coef = [h (k + c), mu].  The last block turns the sums
 // into the coefficients of the next pass (coef_next) or into the final norm.
 //
-// Bound by the FP64 pipe, one FMA lane per clock and SM as measured (an FP64 instruction whose predicate
-// is false costs as much as one whose predicate is true): n (k + c) FMAs per dot pass and per update.  So a
-// thread owns whole rows and nothing is done twice or under a predicate: the update is one FMA per column,
-// the dots go over the columns in batches of eight (then four, two, one) whose accumulators sit in
-// registers, and a batch is reduced once, at the end.  A row's columns are read again by the next
-// batches from L1 / L2.  Measured at n = 1.3 million, 15 columns: dots 66 us (62 us of FMAs); tiles of Q in
-// shared memory with a partial sum per tile and column took 94-107 us.
+// n (k + c) FMAs per dot pass and per update, and an SM starts an FP64 warp instruction every 16 to 19 cycles, also
+// when its predicate is false.  So a thread owns whole rows and nothing is done twice or under a
+// predicate: the update is one FMA per column, the dots go over the columns in batches of eight (then
+// four, two, one) whose accumulators sit in registers, and a batch is reduced once, at the end.
+// Measured at n = 1.3 million: dots of 15 columns 66 us (31 to 37 us of FP64 pipe, 25 us of bytes); tiles of Q
+// in shared memory with a partial sum per tile and column took 94-107 us.  ncu at 12 columns: dots 64 us
+// with the FP64 pipe 60 % busy, update with dots 96 us (71 %), update with norm 92 us (40 %), DRAM at 19 to
+// 33 % of its peak, a quarter of the warp slots filled and most stalls on loads: what is left between the
+// pipe and the time is loads in flight.
 constexpr int kTsBatch = 8;
 
 __device__ __forceinline__ const double* ts_col(const OuterArgs& a, int k, int j) {

@@ -3,9 +3,11 @@
 // The outer loop runs on the host, one synchronisation per outer step (to read
 // ||r|| and the Ritz values written by the device into mapped pinned memory) and
 // one after each orthogonalisation (breakdown test).  Everything that touches an
-// n-vector runs in the kernels of inner_*.cu and outer.cu.  The inner MINRES solve
-// is launched in chunks of iterations; its kernels return at once after the
-// device-side stopping test has fired, so a chunk may end with a few empty launches.
+// n-vector runs in the kernels of inner_*.cu and outer.cu.  An inner MINRES solve is one
+// launch: the cluster kernel of small graphs, or a CUDA graph whose WHILE node holds a few
+// iterations.  Single inner solves enqueue iterations ahead of the device's count, and
+// inner_graph = 0 or event profiling launches them in chunks.  The kernels of an iteration return
+// at once after the device-side stopping test has fired, so each of these may end with empty ones.
 #include <algorithm>
 #include <chrono>
 #include <map>
