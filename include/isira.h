@@ -82,7 +82,8 @@ typedef struct {
     int inner_graph;      /* 1: each inner solve is one CUDA-graph launch whose WHILE node repeats the
                              iteration until the device-side stopping test fires (no host round trip),
                              or, on small graphs without rows above 64 neighbours and with the diagonal
-                             preconditioner, one kernel launch that holds the whole solve;
+                             preconditioner, one kernel launch that holds the whole solve, at the
+                             deflation ranks where that is the faster way (see isira_inner_route);
                              0: chunked launches with a host check after each chunk */
     int reorder;          /* 1: relabel the vertices internally by descending degree (stable), which
                              packs the vectors' entries of high-degree vertices together for cache

@@ -27,6 +27,7 @@ def test_row_limits_and_cta_counts(prec, n, ctas):
 
 @pytest.mark.parametrize("make,prec,ctas,staged", [
     (lambda: sg.erdos_renyi(12347, 8.0, seed=1), "mixed", 16, 1),     # more lines than the copy moves
+    (lambda: sg.erdos_renyi(17000, 8.0, seed=5), "mixed", 16, 1),
     (lambda: sg.grid2d(112, 88), "mixed", 16, 0),                     # fewer
     (lambda: sg.erdos_renyi(12347, 8.0, seed=1), "fp64", 16, 0),
     (lambda: sg.watts_strogatz(79999, 10, 0.1, seed=6), "mixed", 16, 0),
